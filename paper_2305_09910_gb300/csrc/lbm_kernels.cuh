@@ -564,21 +564,6 @@ __device__ __forceinline__ V gelu_v(V a) {
 
 __device__ __forceinline__ float gelu_erf(float a) { return gelu_v<float>(a); }
 
-// erf of the same approximation, for the derivative Phi(x) + x phi(x) of the GELU
-__device__ __forceinline__ float erf_as(float z) {
-  const float a = fabsf(z);
-  const float t = __fdividef(1.f, fmaf(0.3275911f, a, 1.f));
-  float q = fmaf(1.061405429f, t, -1.453152027f);
-  q = fmaf(q, t, 1.421413741f);
-  q = fmaf(q, t, -0.284496736f);
-  q = fmaf(q, t, 0.254829592f);
-  const float r = fmaf(-q * t, ex2_approx(-a * a * 1.4426950408889634f), 1.f);
-  return copysignf(r, z);
-}
-__device__ __forceinline__ float gelu_grad_f(float a) {
-  return 0.5f * (1.f + erf_as(a * 0.70710678118654752f)) + a * 0.39894228040143268f * __expf(-0.5f * a * a);
-}
-
 // Orientation of the +/- pair (I, I+1), I odd: the member whose first non-zero velocity
 // component is positive is the primary one, so that c.u is a plain sum with a leading +.
 __host__ __device__ constexpr int lead(int i) { return cx(i) ? cx(i) : cy(i) ? cy(i) : cz(i); }
