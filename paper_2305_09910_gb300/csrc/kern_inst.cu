@@ -170,20 +170,33 @@ cudaError_t launch_step_mlp(const KParams& p, int mode, cudaStream_t stream, int
   }
 }
 
+// Blocks of k_row_sums.  EX_SUM: one wave of what is resident (8 per SM).  EX_STATS: four times as
+// many, since a block's rows are all of one plane and those of a wall plane take several times as
+// long (256x128x130 channel: 111 us with one wave; four take 25 us off a pass of two steps, sums,
+// statistics and exports).
+#ifndef LBM_ROW_BLOCKS
+#define LBM_ROW_BLOCKS (8 * 152)
+#endif
+
 template <int Q, class S, int PAR>
 static void export_par(const KParams& p, int mode, const ExportArgs& a, const Launch& L) {
-  const dim3 rows((unsigned)p.ny, (unsigned)p.nz);
   switch (mode) {
     case EX_POP: k_export<Q, S, PAR, EX_POP><<<L.grid, L.block, 0, L.stream>>>(p, a); break;
     case EX_MOM: k_export<Q, S, PAR, EX_MOM><<<L.grid, L.block, 0, L.stream>>>(p, a); break;
-    case EX_SUM:
-      k_row_sums<Q, S, PAR, EX_SUM><<<rows, ROW_THREADS, 0, L.stream>>>(p, a.partial);
-      k_row_total<EX_SUM><<<1, 256, 0, L.stream>>>(a.partial, p.ny, p.nz, a.sums);
+    case EX_SUM: {
+      const int rows = p.ny * p.nz, cnt = (rows + LBM_ROW_BLOCKS - 1) / LBM_ROW_BLOCKS;
+      const int nblk = (rows + cnt - 1) / cnt;
+      k_row_sums<Q, S, PAR, EX_SUM><<<(unsigned)nblk, ROW_THREADS, 0, L.stream>>>(p, cnt, a.partial);
+      k_row_total<EX_SUM><<<1, 256, 0, L.stream>>>(a.partial, p.ny, nblk, a.sums);
       break;
-    default:
-      k_row_sums<Q, S, PAR, EX_STATS><<<rows, ROW_THREADS, 0, L.stream>>>(p, a.partial);
-      k_row_total<EX_STATS><<<(unsigned)p.ny, 256, 0, L.stream>>>(a.partial, p.ny, p.nz, a.sums);
+    }
+    default: {
+      const int per = std::max(1, 4 * LBM_ROW_BLOCKS / p.ny);  // blocks per plane
+      const int cnt = (p.nz + per - 1) / per, nblk = (p.nz + cnt - 1) / cnt * p.ny;
+      k_row_sums<Q, S, PAR, EX_STATS><<<(unsigned)nblk, ROW_THREADS, 0, L.stream>>>(p, cnt, a.partial);
+      k_row_total<EX_STATS><<<(unsigned)p.ny, 256, 0, L.stream>>>(a.partial, p.ny, nblk, a.sums);
       break;
+    }
   }
 }
 

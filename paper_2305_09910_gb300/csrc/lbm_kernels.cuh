@@ -232,11 +232,19 @@ __device__ __forceinline__ int face_rank(int t) {
   return t == FACE_WALL ? 4 : t == FACE_INFLOW ? 3 : t == FACE_OUTFLOW ? 2 : 1;
 }
 
+// inverse of (cx, cy, cz) over the 27 velocities: 5 bits per index, 12 to a word
+__host__ __device__ constexpr unsigned long long dir_word(int w) {
+  unsigned long long t = 0;
+  for (int j = 0; j < 27; j++) {
+    const int k = (cx(j) + 1) + 3 * (cy(j) + 1) + 9 * (cz(j) + 1);
+    if (k / 12 == w) t |= (unsigned long long)j << (5 * (k % 12));
+  }
+  return t;
+}
 __device__ __forceinline__ int dir_index(int dx, int dy, int dz) {
-  // inverse of (cx, cy, cz) over the 27 velocities
-  for (int j = 0; j < 27; j++)
-    if (cx(j) == dx && cy(j) == dy && cz(j) == dz) return j;
-  return 0;
+  constexpr unsigned long long w0 = dir_word(0), w1 = dir_word(1), w2 = dir_word(2);
+  const int k = (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1);
+  return (int)((k < 12 ? w0 >> (5 * k) : k < 24 ? w1 >> (5 * (k - 12)) : w2 >> (5 * (k - 24))) & 31);
 }
 
 // Returns the rule for the incoming population i of fluid cell (x,y,z) and, except for
@@ -346,7 +354,12 @@ struct Nbr {
 // ---- loading the pre-collision populations of one cell ---------------------------------
 // PAR 0: natural layout (own slots); 1: AA swapped layout (gather); 2: post-collision values
 // in natural layout (two-grid pull, gather).
-template <int Q, class S, int PAR>
+// BATCH: a boundary cell issues all its loads before it uses a value.  A use after each load (the
+// moving-wall sum) makes them wait for one another, about 10 us for a warp that holds a boundary
+// cell: the sums of a 256x128x130 channel took 329 us that way and 122 us batched.  The step
+// kernels, compiled for more resident warps, spill with it and are slower (D3Q27 tunnel, pull
+// 540 -> 609 us a step).
+template <int Q, class S, int PAR, bool BATCH = false>
 __device__ __forceinline__ void load_state(const KParams& p, int x, int y, int z, int cell, int cls,
                                            float (&f)[Q], unsigned& outmask) {
   outmask = 0;
@@ -379,11 +392,11 @@ __device__ __forceinline__ void load_state(const KParams& p, int x, int y, int z
 #pragma unroll
     for (int i = 0; i < Q; i++) f[i] = ldp<S>(p, plane_ptr<S>(p, PAR == 2 ? i : opp(i)) + nb.src(p, i));
   } else {
-    // boundary cell: the precomputed rules make every load independent of the others
+    // boundary cell: the precomputed rules name the slot of every direction
     const unsigned long long r = rule_at(p, cell);
     Nbr nb;
     nb.init(p, x, y, z);
-    unsigned special = 0;
+    unsigned special = 0, inflow = 0;
 #pragma unroll
     for (int i = 0; i < Q; i++) {
       const int k = (int)((r >> (2 * i)) & 3);
@@ -395,8 +408,14 @@ __device__ __forceinline__ void load_state(const KParams& p, int x, int y, int z
                                  : plane_ptr<S>(p, PAR == 2 ? opp(i) : i) + cell;
       float v = ldp<S>(p, a);
       // moving-wall value rounded like the natural-layout slot that holds it
-      if (k == R_INFLOW) v = rnd<S>(v + p.inflow_term[i]);
+      if (BATCH) inflow |= (k == R_INFLOW ? 1u : 0u) << i;
+      else if (k == R_INFLOW) v = rnd<S>(v + p.inflow_term[i]);
       f[i] = v;
+    }
+    if (BATCH && inflow) {
+#pragma unroll
+      for (int i = 0; i < Q; i++)
+        if (inflow & (1u << i)) f[i] = rnd<S>(f[i] + p.inflow_term[i]);
     }
     if (special) {
 #pragma unroll
@@ -1200,11 +1219,18 @@ __device__ __forceinline__ void stat_warp_store(const KParams& p, int y, int z, 
     p.stats_w[(((long long)z * p.ny + y) * nws + ws) * NSTAT + k + 5 * b4] = s;
 }
 
+// hi + lo += v with the rounding error of the addition carried along (Knuth's TwoSum): hi + lo
+// stays the exact sum up to the rounding of lo, about 2^-48 of it.  FP64 arithmetic is slow on
+// this GPU, so long float32 sums are kept this way and widened once.
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
+  const float s = __fadd_rn(hi, v);
+  const float bp = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(v, bp)));
+  hi = s;
+}
+
 // Plane sums of the sampled statistics: sums[y * 10 + k] += sum over z and the nws warp
-// slots of each row (FP64).  One block per plane y.  A thread sums its slots in FP32 with the
-// rounding error of every addition carried along (Knuth's TwoSum: hi + lo is the exact sum up
-// to the rounding of lo, about 2^-48 of it), then widens hi and lo once: FP64 arithmetic, which
-// is slow on this GPU, is left to the block's final reduction.
+// slots of each row (FP64).  One block per plane y; a thread sums its slots by two_sum.
 static __global__ void __launch_bounds__(256) k_stats_total(const float* stats_w, int ny, int nz, int nws, double* sums) {
   const int y = blockIdx.x;
   float hi[NSTAT], lo[NSTAT];
@@ -1217,12 +1243,7 @@ static __global__ void __launch_bounds__(256) k_stats_total(const float* stats_w
     const float* src = stats_w + (((long long)z * ny + y) * nws + ws) * NSTAT;
 #pragma unroll
     for (int k = 0; k < NSTAT; k++) {
-      const float v = src[k];
-      const float s = __fadd_rn(hi[k], v);
-      const float bp = __fsub_rn(s, hi[k]);
-      const float err = __fadd_rn(__fsub_rn(hi[k], __fsub_rn(s, bp)), __fsub_rn(v, bp));
-      lo[k] = __fadd_rn(lo[k], err);
-      hi[k] = s;
+      two_sum(hi[k], lo[k], src[k]);
     }
   }
   double acc[NSTAT];
@@ -1356,10 +1377,17 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 template <int Q, class S, int PAR, int MODE>
 __global__ void __launch_bounds__(128) k_export(const __grid_constant__ KParams p, ExportArgs a) {
-  LBM_CELL_COORDS
+  const int x = blockIdx.x * 32 + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (y >= p.ny) return;  // whole warp
+  const int cell = cidx(p, x, y, z);
   float f[Q];
-  unsigned outmask;
-  load_state<Q, S, PAR>(p, x, y, z, cell, cls, f, outmask);
+  unsigned outmask = 0;
+  const bool early = PAR != 0 && off_faces(p, x, y, z);
+  if (early) gather_interior<Q, S, PAR>(p, cell, f);  // in flight with the class load below
+  const int cls = x < p.nx ? cls_at(p, cell) : CLS_SKIP;
+  if (!(early && cls == CLS_INTERIOR)) load_state<Q, S, PAR, true>(p, x, y, z, cell, cls, f, outmask);
   outflow_fix<Q>(p, x, f, outmask);
   const bool fluid = cls != CLS_SKIP;
   const long long dense = ((long long)z * p.ny + y) * p.nx + x;
@@ -1384,54 +1412,79 @@ __global__ void __launch_bounds__(128) k_export(const __grid_constant__ KParams 
   }
 }
 
-// Sums over fluid cells, in two passes.  k_row_sums: one block per (y, z) row; a thread adds
-// the values of its few cells of the row in FP32, the block adds the threads' partials in
-// FP64 and writes partial[(z ny + y) K + k].  k_row_total then adds the rows in FP64:
+// Sums over fluid cells, in two passes.  k_row_sums: a block takes `cnt` rows, its warps the
+// 32-cell segments of these in turn; a lane sums its cells by two_sum, a warp its lanes likewise, and
+// the block's warps in FP64 go to partial[block K + k].  k_row_total then adds the blocks in FP64:
 //   EX_SUM   (K = 5: count, drho, j_x, j_y, j_z) -> sums[0] = count + sum drho = sum rho,
 //            sums[1..3] = sum j = sum rho u (j includes F/2, so u = j / rho);
 //   EX_STATS (K = 10: count, u_x, u_y, u_z, u_x^2, u_y^2, u_z^2, u_x u_y, u_x u_z, u_y u_z)
-//            -> sums[y * 10 + k] += sum over the x-z plane y.
+//            -> sums[y * 10 + k] += sum over the x-z plane y; the block's rows are then rows of
+//            plane y = block % ny.
+// Bound by HBM (one read of the state).  FP64 runs at 1/64 of the FP32 rate here: ten FP64 warp
+// reductions per warp took as long as reading ten rows, hence two_sum and one wave of blocks.
+// 256x128x130 D3Q19 FP32 after a step, both passes: EX_SUM 192 -> 70 us, EX_STATS 275 -> under 118
+// us (before: a block per row, and one block over 16,640 rows in the second pass); read time 48 us.
 template <int MODE>
 __host__ __device__ constexpr int row_k() { return MODE == EX_SUM ? 5 : 10; }
 
 constexpr int ROW_THREADS = 128;
 
 template <int Q, class S, int PAR, int MODE>
-__global__ void __launch_bounds__(ROW_THREADS) k_row_sums(const __grid_constant__ KParams p, double* partial) {
+__global__ void __launch_bounds__(ROW_THREADS, 8) k_row_sums(const __grid_constant__ KParams p, int cnt, double* partial) {
   constexpr int K = row_k<MODE>();
   constexpr int NW = ROW_THREADS / 32;
-  const int y = blockIdx.x, z = blockIdx.y;
-  const int warp = threadIdx.x >> 5;
-  float acc[K];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wpr = p.nxp / 32;
+  const int rows = p.ny * p.nz;
+  // rows row0, row0 + rstep, ... of the lattice (row = z ny + y)
+  const int row0 = MODE == EX_STATS ? (blockIdx.x / p.ny) * cnt * p.ny + blockIdx.x % p.ny : blockIdx.x * cnt;
+  const int rstep = MODE == EX_STATS ? p.ny : 1;
+  float hi[K], lo[K];
 #pragma unroll
-  for (int k = 0; k < K; k++) acc[k] = 0.f;
-  for (int xb = 0; xb < p.nxp; xb += ROW_THREADS) {
-    if (xb + warp * 32 >= p.nxp) break;  // warp-uniform (nxp is a multiple of 32)
-    const int x = xb + threadIdx.x;
+  for (int k = 0; k < K; k++) hi[k] = lo[k] = 0.f;
+  int i = warp / wpr, xw = warp - i * wpr;  // row of the block, segment of the row
+  const int di = NW / wpr, dx = NW - di * wpr;
+  while (i < cnt && row0 + i * rstep < rows) {
+    const int row = row0 + i * rstep;
+    const int z = row / p.ny, y = row - z * p.ny, x = xw * 32 + lane;
+    i += di;
+    xw += dx;
+    if (xw >= wpr) {
+      xw -= wpr;
+      i++;
+    }
     const int cell = cidx(p, x, y, z);
-    const int cls = x < p.nx ? cls_at(p, cell) : CLS_SKIP;
     float f[Q];
-    unsigned outmask;
-    load_state<Q, S, PAR>(p, x, y, z, cell, cls, f, outmask);
+    unsigned outmask = 0;
+    const bool early = PAR != 0 && off_faces(p, x, y, z);
+    if (early) gather_interior<Q, S, PAR>(p, cell, f);  // in flight with the class load below
+    const int cls = x < p.nx ? cls_at(p, cell) : CLS_SKIP;
+    if (!(early && cls == CLS_INTERIOR)) load_state<Q, S, PAR, true>(p, x, y, z, cell, cls, f, outmask);
     outflow_fix<Q>(p, x, f, outmask);
     if (cls == CLS_SKIP) continue;
     const Mom<Q> m = moments<Q>(p, f);
     if (MODE == EX_SUM) {
       const float v[5] = {1.f, m.drho, m.jx, m.jy, m.jz};
 #pragma unroll
-      for (int k = 0; k < K; k++) acc[k] += v[k];
+      for (int k = 0; k < K; k++) two_sum(hi[k], lo[k], v[k]);
     } else {
       const float v[10] = {1.f, m.ux, m.uy, m.uz, m.ux * m.ux, m.uy * m.uy, m.uz * m.uz,
                            m.ux * m.uy, m.ux * m.uz, m.uy * m.uz};
 #pragma unroll
-      for (int k = 0; k < K; k++) acc[k] += v[k];
+      for (int k = 0; k < K; k++) two_sum(hi[k], lo[k], v[k]);
     }
   }
   __shared__ double red[K][NW];
 #pragma unroll
   for (int k = 0; k < K; k++) {
-    const double v = warp_sum((double)acc[k]);
-    if ((threadIdx.x & 31) == 0) red[k][warp] = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_down_sync(0xffffffffu, hi[k], o), l = __shfl_down_sync(0xffffffffu, lo[k], o);
+      two_sum(hi[k], lo[k], h);
+      lo[k] = __fadd_rn(lo[k], l);
+    }
+    // (after an infinity in the sum lo is NaN and hi is the float32 sum)
+    if (lane == 0) red[k][warp] = isfinite(hi[k]) ? (double)hi[k] + (double)lo[k] : (double)hi[k];
   }
   __syncthreads();
   if (threadIdx.x < K) {
@@ -1439,29 +1492,21 @@ __global__ void __launch_bounds__(ROW_THREADS) k_row_sums(const __grid_constant_
     double t = 0.0;
 #pragma unroll
     for (int w = 0; w < NW; w++) t += red[k][w];
-    partial[((long long)z * p.ny + y) * K + k] = t;
+    partial[(long long)blockIdx.x * K + k] = t;
   }
 }
 
-// EX_STATS: one block per plane y (its nz rows); EX_SUM: one block for all rows.
+// EX_STATS: one block per plane y (its nblk / ny blocks); EX_SUM: one block for all of them.
 template <int MODE>
-__global__ void __launch_bounds__(256) k_row_total(const double* partial, int ny, int nz, double* sums) {
+__global__ void __launch_bounds__(256) k_row_total(const double* partial, int ny, int nblk, double* sums) {
   constexpr int K = row_k<MODE>();
   double acc[K];
 #pragma unroll
   for (int k = 0; k < K; k++) acc[k] = 0.0;
-  if (MODE == EX_STATS) {
-    const int y = blockIdx.x;
-    for (int z = threadIdx.x; z < nz; z += blockDim.x) {
+  const int first = MODE == EX_STATS ? blockIdx.x : 0, step = MODE == EX_STATS ? ny : 1;
+  for (int b = first + threadIdx.x * step; b < nblk; b += blockDim.x * step) {
 #pragma unroll
-      for (int k = 0; k < K; k++) acc[k] += partial[((long long)z * ny + y) * K + k];
-    }
-  } else {
-    const long long nrow = (long long)ny * nz;
-    for (long long r = threadIdx.x; r < nrow; r += blockDim.x) {
-#pragma unroll
-      for (int k = 0; k < K; k++) acc[k] += partial[r * K + k];
-    }
+    for (int k = 0; k < K; k++) acc[k] += partial[(long long)b * K + k];
   }
   __shared__ double red[K][8];
 #pragma unroll
@@ -1516,8 +1561,11 @@ __global__ void __launch_bounds__(128) k_set_pop(const __grid_constant__ KParams
   const long long dense = ((long long)z * p.ny + y) * p.nx + x;
   const long long N = (long long)p.nx * p.ny * p.nz;
   const bool fluid = cls != CLS_SKIP;
+  float f[Q];  // all loads first: a store may alias df as far as the compiler knows, and would hold them back
 #pragma unroll
-  for (int i = 0; i < Q; i++) stp<S>(p, plane_ptr<S>(p, i) + cell, fluid ? df[i * N + dense] : 0.f);
+  for (int i = 0; i < Q; i++) f[i] = df[i * N + dense];
+#pragma unroll
+  for (int i = 0; i < Q; i++) stp<S>(p, plane_ptr<S>(p, i) + cell, fluid ? f[i] : 0.f);
 }
 
 }  // namespace lbm
