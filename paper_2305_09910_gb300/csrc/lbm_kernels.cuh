@@ -157,6 +157,9 @@ __device__ __forceinline__ bool chk(const KParams& p, const void* a, int bytes, 
 __device__ __forceinline__ int cls_at(const KParams& p, long long cell) {
   return chk(p, p.cls + cell, 1, CHK_CLS) ? (p.cls[cell] & CLS_MASK) : CLS_SKIP;
 }
+__device__ __forceinline__ int cls_byte(const KParams& p, long long cell) {  // with CLS_XFACE
+  return chk(p, p.cls + cell, 1, CHK_CLS) ? p.cls[cell] : CLS_SKIP;
+}
 __device__ __forceinline__ int flag_at(const KParams& p, long long cell) {
   return chk(p, p.flags + cell, 1, CHK_FLAGS) ? p.flags[cell] : CELL_SOLID;
 }
@@ -351,6 +354,115 @@ struct Nbr {
   }
 };
 
+// ---- boundary cells: the slot of an incoming population ----------------------------------
+// Resolved inline, direction by direction, from the cell's rule word and three reflection tests
+// per axis: the loop over calls that it replaces made the AA odd and pull steps keep their
+// populations across calls (44 to 144 bytes of spills) and took a warp with a free-slip cell tens
+// of microseconds.  With gather_xface, 375x190x187 D3Q27 FP32 tunnel: AA odd 865 -> 543 us, pull
+// 540 -> 475 us; 512x256x256 D3Q19 FP32 channel: AA odd 896 -> 825 us, pull 775 -> 770 us.
+// Direction i with the axes of `sel` reflected (bit 0 x, 1 y, 2 z), 5 bits per sel.
+template <int I>
+struct Reflected {
+  static constexpr unsigned long long word() {
+    unsigned long long w = 0;
+    for (int sel = 0; sel < 8; sel++)
+      for (int j = 0; j < 27; j++)
+        if (cx(j) == (sel & 1 ? -cx(I) : cx(I)) && cy(j) == (sel & 2 ? -cy(I) : cy(I)) &&
+            cz(j) == (sel & 4 ? -cz(I) : cz(I)))
+          w |= (unsigned long long)j << (5 * sel);
+    return w;
+  }
+  static constexpr unsigned long long w = word();
+};
+
+// The rules of one boundary cell, with what its directions share.
+struct BoundaryCell {
+  unsigned long long r;
+  Nbr nb;
+  int x, y, z, cell;
+  unsigned refl;  // bit c + 1 + 3 axis: the source of velocity component c = -1, 1 is reflected (free-slip)
+  bool outflow;   // on the zero-gradient face: R_SPECIAL with c_x = -1 copies the upstream cell's
+  __device__ __forceinline__ void init(const KParams& p, int x_, int y_, int z_, int cell_) {
+    r = rule_at(p, cell_);
+    nb.init(p, x_, y_, z_);
+    x = x_;
+    y = y_;
+    z = z_;
+    cell = cell_;
+    refl = 0;
+    const int xc[3] = {x, y, z}, n[3] = {p.nx, p.ny, p.nz};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      if (xc[a] == 0 && p.face[2 * a] != FACE_PERIODIC && p.face[2 * a] != FACE_HALO) refl |= 4u << (3 * a);
+      if (xc[a] == n[a] - 1 && p.face[2 * a + 1] != FACE_PERIODIC && p.face[2 * a + 1] != FACE_HALO) refl |= 1u << (3 * a);
+    }
+    outflow = p.outflow && x == p.nx - 1;
+  }
+};
+
+// The slot (address in the state array) that holds the incoming population I of a boundary cell,
+// PAR as in load_state; returns its rule, R_SPECIAL only for an outflow copy (which has no slot).
+template <int I, class S, int PAR>
+__device__ __forceinline__ int boundary_slot(const KParams& p, const BoundaryCell& b, S*& a) {
+  int k = (int)((b.r >> (2 * I)) & 3);
+  if (k == R_BB || k == R_INFLOW) {
+    a = plane_ptr<S>(p, PAR == 2 ? opp(I) : I) + b.cell;
+  } else if (k == R_STREAM) {
+    a = plane_ptr<S>(p, PAR == 2 ? I : opp(I)) + b.nb.src(p, I);
+  } else if (!(b.outflow && cx(I) == -1)) {
+    const bool fx = cx(I) && (b.refl >> (cx(I) + 1)) & 1, fy = cy(I) && (b.refl >> (cy(I) + 4)) & 1,
+               fz = cz(I) && (b.refl >> (cz(I) + 7)) & 1;
+    const int j = (int)((Reflected<I>::w >> (5 * ((fx ? 1 : 0) | (fy ? 2 : 0) | (fz ? 4 : 0)))) & 31);
+    const int src = ((fz ? b.z : b.nb.zs[cz(I) + 1]) * p.ny + (fy ? b.y : b.nb.ys[cy(I) + 1])) * p.nxp +
+                    (fx ? b.x : b.nb.xs[cx(I) + 1]);
+    a = plane_ptr<S>(p, PAR == 2 ? j : opp(j)) + src;
+    k = R_STREAM;
+  }
+  return k;
+}
+
+template <int Q, class S, int PAR, bool BATCH, int... I>
+__device__ __forceinline__ void boundary_loads(const KParams& p, const BoundaryCell& b, float (&f)[Q], unsigned& outmask,
+                                               std::integer_sequence<int, I...>) {
+  unsigned inflow = 0;
+  auto one = [&](auto I_) {
+    constexpr int i = decltype(I_)::value;
+    S* a;
+    const int k = boundary_slot<i, S, PAR>(p, b, a);
+    if (k == R_SPECIAL) {
+      outmask |= 1u << i;
+      return;
+    }
+    float v = ldp<S>(p, a);
+    // moving-wall value rounded like the natural-layout slot that holds it
+    if (BATCH) inflow |= (k == R_INFLOW ? 1u : 0u) << i;
+    else if (k == R_INFLOW) v = rnd<S>(v + p.inflow_term[i]);
+    f[i] = v;
+  };
+  (one(std::integral_constant<int, I>{}), ...);
+  if (BATCH && inflow) {
+#pragma unroll
+    for (int i = 0; i < Q; i++)
+      if (inflow & (1u << i)) f[i] = rnd<S>(f[i] + p.inflow_term[i]);
+  }
+}
+
+// AA odd: f*_opp(i) goes back into the slot f_i came from (none for an outflow copy).
+template <int Q, class S, int... I>
+__device__ __forceinline__ void boundary_stores(const KParams& p, const BoundaryCell& b, const float (&fs)[Q],
+                                                std::integer_sequence<int, I...>) {
+  auto one = [&](auto I_) {
+    constexpr int i = decltype(I_)::value;
+    S* a;
+    const int k = boundary_slot<i, S, 1>(p, b, a);
+    if (k == R_SPECIAL) return;
+    float v = fs[opp(i)];
+    if (k == R_INFLOW) v = rnd<S>(v) + p.inflow_term[i];  // same rounding as the swapped path
+    stp<S>(p, a, v);
+  };
+  (one(std::integral_constant<int, I>{}), ...);
+}
+
 // ---- loading the pre-collision populations of one cell ---------------------------------
 // PAR 0: natural layout (own slots); 1: AA swapped layout (gather); 2: post-collision values
 // in natural layout (two-grid pull, gather).
@@ -393,39 +505,9 @@ __device__ __forceinline__ void load_state(const KParams& p, int x, int y, int z
     for (int i = 0; i < Q; i++) f[i] = ldp<S>(p, plane_ptr<S>(p, PAR == 2 ? i : opp(i)) + nb.src(p, i));
   } else {
     // boundary cell: the precomputed rules name the slot of every direction
-    const unsigned long long r = rule_at(p, cell);
-    Nbr nb;
-    nb.init(p, x, y, z);
-    unsigned special = 0, inflow = 0;
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const int k = (int)((r >> (2 * i)) & 3);
-      if (k == R_SPECIAL) {
-        special |= 1u << i;
-        continue;
-      }
-      const S* a = k == R_STREAM ? plane_ptr<S>(p, PAR == 2 ? i : opp(i)) + nb.src(p, i)
-                                 : plane_ptr<S>(p, PAR == 2 ? opp(i) : i) + cell;
-      float v = ldp<S>(p, a);
-      // moving-wall value rounded like the natural-layout slot that holds it
-      if (BATCH) inflow |= (k == R_INFLOW ? 1u : 0u) << i;
-      else if (k == R_INFLOW) v = rnd<S>(v + p.inflow_term[i]);
-      f[i] = v;
-    }
-    if (BATCH && inflow) {
-#pragma unroll
-      for (int i = 0; i < Q; i++)
-        if (inflow & (1u << i)) f[i] = rnd<S>(f[i] + p.inflow_term[i]);
-    }
-    if (special) {
-#pragma unroll
-      for (int i = 0; i < Q; i++) {
-        if (!(special & (1u << i))) continue;
-        int pl, ce;
-        if (resolve_special(p, x, y, z, i, pl, ce) == K_OUTCOPY) outmask |= 1u << i;
-        else f[i] = ldp<S>(p, plane_ptr<S>(p, PAR == 2 ? opp(pl) : pl) + ce);
-      }
-    }
+    BoundaryCell b;
+    b.init(p, x, y, z, cell);
+    boundary_loads<Q, S, PAR, BATCH>(p, b, f, outmask, std::make_integer_sequence<int, Q>{});
   }
 }
 
@@ -442,6 +524,42 @@ template <int Q, class S, int PAR>
 __device__ __forceinline__ void gather_interior(const KParams& p, int cell, float (&f)[Q]) {
 #pragma unroll
   for (int i = 0; i < Q; i++) f[i] = ldg_pop<S>(p, static_cast<const S*>(PAR == 2 ? p.gb[i] : p.ga[i]) + cell);
+}
+
+// Gather of a simple inflow (x = 0) or outflow (x = nx - 1) face cell (CLS_XFACE), PAR 1 or 2: the
+// directions crossing the face come from the own cell with the moving-wall term, or are left to
+// outflow_fix; all others stream as in an interior cell.  Every load is issued before a value is
+// used: a warp that holds one such lane (two of every row) waits for memory once more, not per direction.
+template <int Q, class S, int PAR>
+__device__ __forceinline__ void gather_xface(const KParams& p, int x, int cell, float (&f)[Q], unsigned& outmask) {
+  const bool in = x == 0;
+#pragma unroll
+  for (int i = 0; i < Q; i++) {
+    const S* a = static_cast<const S*>(PAR == 2 ? p.gb[i] : p.ga[i]) + cell;
+    if (cx(i) == 1 && in) a = plane_ptr<S>(p, PAR == 2 ? opp(i) : i) + cell;
+    f[i] = cx(i) == -1 && !in ? 0.f : ldp<S>(p, a);
+  }
+#pragma unroll
+  for (int i = 0; i < Q; i++) {
+    if (cx(i) == 1 && in) f[i] = rnd<S>(f[i] + p.inflow_term[i]);
+    if (cx(i) == -1 && !in) outmask |= 1u << i;
+  }
+}
+
+// AA odd stores of such a cell: back into the slots of gather_xface.
+template <int Q, class S>
+__device__ __forceinline__ void store_xface(const KParams& p, int x, int cell, const float (&fs)[Q]) {
+  const bool in = x == 0;
+#pragma unroll
+  for (int i = 0; i < Q; i++) {
+    S* a = static_cast<S*>(p.ga[i]) + cell;
+    float v = fs[opp(i)];
+    if (cx(i) == 1 && in) {
+      a = plane_ptr<S>(p, i) + cell;
+      v = rnd<S>(v) + p.inflow_term[i];
+    }
+    if (!(cx(i) == -1 && !in)) stp<S>(p, a, v);
+  }
 }
 
 // Zero-gradient outflow: lane x = nx-1 takes the incoming c_x = -1 populations of lane x-1.
@@ -484,23 +602,9 @@ __device__ __forceinline__ void store_state(const KParams& p, int x, int y, int 
 #pragma unroll
     for (int i = 0; i < Q; i++) stp<S>(p, plane_ptr<S>(p, opp(i)) + nb.src(p, i), fs[opp(i)]);
   } else {
-    const unsigned long long r = rule_at(p, cell);
-    Nbr nb;
-    nb.init(p, x, y, z);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const int k = (int)((r >> (2 * i)) & 3);
-      int pl = opp(i), ce = nb.src(p, i);
-      if (k == R_BB || k == R_INFLOW) {
-        pl = i;
-        ce = cell;
-      } else if (k == R_SPECIAL) {
-        if (resolve_special(p, x, y, z, i, pl, ce) == K_OUTCOPY) continue;
-      }
-      float v = fs[opp(i)];
-      if (k == R_INFLOW) v = rnd<S>(v) + p.inflow_term[i];  // same rounding as the swapped path
-      stp<S>(p, plane_ptr<S>(p, pl) + ce, v);
-    }
+    BoundaryCell b;
+    b.init(p, x, y, z, cell);
+    boundary_stores<Q, S>(p, b, fs, std::make_integer_sequence<int, Q>{});
   }
 }
 
@@ -1290,8 +1394,11 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? 8 : LBM_STEP_MINB1
   unsigned outmask = 0;
   const bool early = LOAD != 0 && off_faces(p, x, y, z);
   if (early) gather_interior<Q, S, LOAD>(p, cell, f);  // in flight with the class load below
-  const int cls = x < p.nx ? cls_at(p, cell) : CLS_SKIP;
-  if (!(early && cls == CLS_INTERIOR)) load_state<Q, S, LOAD>(p, x, y, z, cell, cls, f, outmask);
+  const int cbyte = x < p.nx ? cls_byte(p, cell) : CLS_SKIP;
+  const int cls = cbyte & CLS_MASK;
+  const bool xface = LOAD != 0 && (cbyte & CLS_XFACE);
+  if (LOAD != 0 && xface) gather_xface<Q, S, LOAD == 0 ? 1 : LOAD>(p, x, cell, f, outmask);
+  else if (!(early && cls == CLS_INTERIOR)) load_state<Q, S, LOAD>(p, x, y, z, cell, cls, f, outmask);
   outflow_fix<Q>(p, x, f, outmask);
   if (!STATS && cls == CLS_SKIP) return;
   float v[NSTAT];
@@ -1301,7 +1408,8 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? 8 : LBM_STEP_MINB1
     Macro<float> M;
     const float rho = collide<Q, CL, float, acc_form<S>, COLL>(p, f, STATS ? &M : nullptr);
     if (!(rho > 0.f && rho < 3.0e38f)) atomicOr(p.status, 1);
-    store_state<Q, S, STORE>(p, x, y, z, cell, cls, f);
+    if (STORE == 1 && xface) store_xface<Q, S>(p, x, cell, f);
+    else store_state<Q, S, STORE>(p, x, y, z, cell, cls, f);
     if (STATS) stat_values(M, v);
   }
   if (STATS) stat_warp_store(p, y, z, blockIdx.x, p.nxp / 32, v);
@@ -1422,7 +1530,7 @@ __global__ void __launch_bounds__(128) k_export(const __grid_constant__ KParams 
 //            plane y = block % ny.
 // Bound by HBM (one read of the state).  FP64 runs at 1/64 of the FP32 rate here: ten FP64 warp
 // reductions per warp took as long as reading ten rows, hence two_sum and one wave of blocks.
-// 256x128x130 D3Q19 FP32 after a step, both passes: EX_SUM 192 -> 70 us, EX_STATS 275 -> under 118
+// 256x128x130 D3Q19 FP32 after a step, both passes: EX_SUM 192 -> 70 us, EX_STATS 275 -> 95
 // us (before: a block per row, and one block over 16,640 rows in the second pass); read time 48 us.
 template <int MODE>
 __host__ __device__ constexpr int row_k() { return MODE == EX_SUM ? 5 : 10; }
