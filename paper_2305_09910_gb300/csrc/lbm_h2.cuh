@@ -103,14 +103,14 @@ __device__ __noinline__ void pair_fallback(const KParams& p, int x, int y, int z
   if (clsA != CLS_SKIP) {
     Macro<float> M;
     const float r = collide<Q, CL, float, false>(p, fa, STATS ? &M : nullptr);
-    if (!(r > 0.f && r < 3.0e38f)) atomicOr(p.status, 1);
+    if (!(r > 0.f && r < 3.0e38f)) flag_unstable(p);
     store_state<Q, S, STORE>(p, x, y, z, cell, clsA, fa);
     if (STATS) stat_values(M, v);
   }
   if (clsB != CLS_SKIP) {
     Macro<float> M;
     const float r = collide<Q, CL, float, false>(p, fb, STATS ? &M : nullptr);
-    if (!(r > 0.f && r < 3.0e38f)) atomicOr(p.status, 1);
+    if (!(r > 0.f && r < 3.0e38f)) flag_unstable(p);
     store_state<Q, S, STORE>(p, x + 1, y, z, cell + 1, clsB, fb);
     if (STATS) {
       float w[NSTAT];
@@ -283,7 +283,7 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
   const bool liveA = SPLIT ? (clsA == CLS_INTERIOR || xfA) : clsA != CLS_SKIP;
   const bool liveB = SPLIT ? (clsB == CLS_INTERIOR || xfB) : clsB != CLS_SKIP;
   if ((liveA && !(rho.x > 0.f && rho.x < 3.0e38f)) || (liveB && !(rho.y > 0.f && rho.y < 3.0e38f)))
-    atomicOr(p.status, 1);
+    flag_unstable(p);
   if (STATS) {
     float va[NSTAT], vb[NSTAT];
     Macro<float> Ma, Mb;
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
 #pragma unroll
     for (int i = 0; i < Q; i++) h[i] = __byte_perm(h[i], bits16<S>(f[i]), 0x5410);
 #endif
-    if (!(ra > 0.f && ra < 3.0e38f) || !(rb > 0.f && rb < 3.0e38f)) atomicOr(p.status, 1);
+    if (!(ra > 0.f && ra < 3.0e38f) || !(rb > 0.f && rb < 3.0e38f)) flag_unstable(p);
 #pragma unroll
     for (int i = 0; i < Q; i++) {
       if (STORE == 0) {
@@ -510,7 +510,7 @@ __device__ __noinline__ void list_cell(const KParams& p, long long t) {
     f[i] = v;
   }
   const float rho = collide<Q, CL, float, acc_form<S>>(p, f, nullptr);
-  if (!(rho > 0.f && rho < 3.0e38f)) atomicOr(p.status, 1);
+  if (!(rho > 0.f && rho < 3.0e38f)) flag_unstable(p);
   store_state<Q, S, 2>(p, 0, 0, 0, cell, CLS_BOUNDARY, f);
 }
 

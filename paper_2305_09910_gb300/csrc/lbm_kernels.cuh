@@ -167,6 +167,13 @@ __device__ __forceinline__ unsigned long long rule_at(const KParams& p, long lon
   return chk(p, p.rules + cell, 8, CHK_RULES) ? p.rules[cell] : 0ull;
 }
 
+// Sets the instability bit.  The bit is read first: in a run that has diverged every cell comes
+// here, and an atomic per cell on one address took a quarter of a D3Q27 step (375x190x187 AA tunnel
+// after it diverged, ten steps and the moments: 7.23 -> 5.16 ms).  A stale 0 only costs one more atomic.
+__device__ __forceinline__ void flag_unstable(const KParams& p) {
+  if (!(*p.status & 1)) atomicOr(p.status, 1);
+}
+
 __device__ __forceinline__ int cidx(const KParams& p, int x, int y, int z) {
   return (z * p.ny + y) * p.nxp + x;
 }
@@ -1407,7 +1414,7 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? 8 : LBM_STEP_MINB1
   if (cls != CLS_SKIP) {
     Macro<float> M;
     const float rho = collide<Q, CL, float, acc_form<S>, COLL>(p, f, STATS ? &M : nullptr);
-    if (!(rho > 0.f && rho < 3.0e38f)) atomicOr(p.status, 1);
+    if (!(rho > 0.f && rho < 3.0e38f)) flag_unstable(p);
     if (STORE == 1 && xface) store_xface<Q, S>(p, x, cell, f);
     else store_state<Q, S, STORE>(p, x, y, z, cell, cls, f);
     if (STATS) stat_values(M, v);
@@ -1443,7 +1450,7 @@ __device__ __forceinline__ void step_tile(const KParams& p, int tile) {
   outflow_fix<Q>(p, x, f, outmask);
   if (cls == CLS_SKIP) return;
   const float rho = collide<Q, CL, float, acc_form<S>, COLL>(p, f, nullptr);
-  if (!(rho > 0.f && rho < 3.0e38f)) atomicOr(p.status, 1);
+  if (!(rho > 0.f && rho < 3.0e38f)) flag_unstable(p);
   store_state<Q, S, STORE>(p, x, y, z, cell, cls, f);
 }
 

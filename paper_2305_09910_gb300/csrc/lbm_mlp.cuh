@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(128 * MLP_NG, 1) k_step_mlp(const __grid_const
     les_rates(p, M.qn, M.inv, cs2, wp, wm);
     relax<Q, float, acc_form<S>>(p, f, M, wp, wm);
     if (cls != CLS_SKIP) {
-      if (!(M.rho > 0.f && M.rho < 3.0e38f)) atomicOr(p.status, 1);
+      if (!(M.rho > 0.f && M.rho < 3.0e38f)) flag_unstable(p);
       store_state<Q, S, STORE>(p, x, y, z, cell, cls, f);
     }
     // the next tile's layer-1 MMA overwrites these TMEM columns: order this lane's reads first
