@@ -249,10 +249,10 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const float* rho, const float* u, 
  * rules, fused into one sweep over the lattice per step (the stream-collide kernel of Sec. 3
  * and 5.2, bounded by memory bandwidth).  Asynchronous: returns
  * after enqueuing; instability is reported by lbm_sync.  Once the state is steady, several
- * steps go into one launch: on small lattices (up to 2^17 padded cells for two-grid pull,
- * 2^15 for AA) cooperative launches of up to 4096 steps separated by grid-wide barriers,
- * above that, up to 2^22 padded cells, replays of a CUDA graph of 8 steps, and single
- * launches on larger lattices; the result has the bits of n single steps.
+ * steps go into one launch: on small lattices (for D3Q19 about 155,000 cells in AA and 310,000
+ * in two-grid pull, half of that for D3Q27) cooperative launches of up to 4096 steps separated
+ * by grid-wide barriers, above that, up to 2^22 padded cells, replays of a CUDA graph of 8
+ * steps, and single launches on larger lattices; the result has the bits of n single steps.
  * LBM_ECUDA on a handle that lbm_sync has declared unusable. */
 lbm_status lbm_step(lbm_handle h, int64_t n);
 
@@ -263,7 +263,8 @@ lbm_status lbm_step(lbm_handle h, int64_t n);
  * the step then waited again, with a longer bound, for the tensor core to finish and completed
  * its tiles); or that second wait gave up as well, after which the tensor-core work may still
  * have been running when the results were read and the kernel left: the handle is then marked
- * unusable and every later step returns LBM_ECUDA; or, in a library built with
+ * unusable and every later step returns LBM_ECUDA (likewise when a multi-step launch gave up a
+ * bounded wait for its own blocks); or, in a library built with
  * LBM_BOUNDS_CHECK (liblbm_check.so), a kernel skipped an access outside its array. */
 lbm_status lbm_sync(lbm_handle h);
 

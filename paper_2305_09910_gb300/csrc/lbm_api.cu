@@ -31,6 +31,7 @@ struct lbm_s {
   uint8_t* cls = nullptr;     // cell classes, padded layout
   unsigned long long* rules = nullptr;  // per-direction rules of boundary cells, padded layout
   int* status = nullptr;      // device status word
+  unsigned* arrivals = nullptr; // barrier arrivals of k_step_multi
   int* chk_bad = nullptr;     // first out-of-range access seen by a bounds-checked build
   int* status_host = nullptr; // pinned copy
   double* sums = nullptr;     // 4 doubles (lbm_reduce)
@@ -377,9 +378,9 @@ static cudaError_t dispatch_multi(const lbm_s* h, const KParams& p0, const KPara
   const int odd0 = aa ? h->parity : 0;
   const int cl = h->prm.closure, coll = h->prm.collision;
   switch (h->prm.precision) {
-    case LBM_F32: return launch_step_multi<Q, float>(p0, p1, cl, coll, aa, odd0, nsteps, h->stream, h->nsm);
-    case LBM_F16_SHIFTED: return launch_step_multi<Q, __half>(p0, p1, cl, coll, aa, odd0, nsteps, h->stream, h->nsm);
-    default: return launch_step_multi<Q, __nv_bfloat16>(p0, p1, cl, coll, aa, odd0, nsteps, h->stream, h->nsm);
+    case LBM_F32: return launch_step_multi<Q, float>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
+    case LBM_F16_SHIFTED: return launch_step_multi<Q, __half>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
+    default: return launch_step_multi<Q, __nv_bfloat16>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
   }
 }
 
@@ -538,6 +539,7 @@ lbm_status lbm_destroy(lbm_handle h) {
   if (h->cls) cudaFreeAsync(h->cls, h->stream);
   if (h->rules) cudaFreeAsync(h->rules, h->stream);
   if (h->status) cudaFreeAsync(h->status, h->stream);
+  if (h->arrivals) cudaFreeAsync(h->arrivals, h->stream);
   if (h->chk_bad) cudaFreeAsync(h->chk_bad, h->stream);
   if (h->sums) cudaFreeAsync(h->sums, h->stream);
   if (h->partial) cudaFreeAsync(h->partial, h->stream);
@@ -641,6 +643,7 @@ lbm_status lbm_create(int nx, int ny, int nz, int stencil, double tau, const lbm
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->cls, (size_t)plane, h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->rules, (size_t)plane * 8, h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->status, sizeof(int), h->stream);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->arrivals, sizeof(unsigned), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->chk_bad, sizeof(int), h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->chk_bad, 0, sizeof(int), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->sums, 4 * sizeof(double), h->stream);
@@ -912,17 +915,22 @@ static bool graph_ready(lbm_handle h) {
 // ---- several steps per launch on small lattices ---------------------------------------------
 // On small lattices the steps are launch-bound even as graph replays: lbm_step runs them as
 // cooperative launches of k_step_multi, MULTI_CHUNK steps at most each, once the state is
-// steady (as for the graphs).  Measured on GB300 (FP32 D3Q19, us per step, multi / graph):
-// pull 32^3 3.8 / 6.7, 64x32x32 4.6 / 7.7, 64^3 11.1 / 11.3, 128x64x64 17.6 / 16.9; AA 32^3
-// 5.1 / 5.6, 64x32x32 6.1 / 6.2, 64^3 14.2 / 10.0 (the AA graph keeps the one array in L2).
-// Hence the limits in padded cells below.  A device that refuses the cooperative launch falls
-// back to the graphs.
-#ifndef LBM_MULTI_MAX_CELLS
-#define LBM_MULTI_MAX_CELLS (1ll << 17)
-#endif
-#ifndef LBM_MULTI_MAX_CELLS_AA
-#define LBM_MULTI_MAX_CELLS_AA (1ll << 15)
-#endif
+// steady (as for the graphs).  The line, in row segments of 32 cells against the warps that are
+// resident at once (cap: 32 per SM for D3Q19, 16 for D3Q27, by registers): AA up to one segment
+// per warp (above that the graph's own-cell steps keep the one array in L2 just as well), pull up
+// to two.  Half storage with the split pull step: a quarter, as its graphs run the x-pair kernel.
+// Measured on GB300 (us per step, multi / graph): D3Q19 FP32 AA 64x32x32 4.5 / 6.0, 96x48x32
+// 6.4 / 7.6, 128x48x32 9.6 / 8.7, 64^3 11.4 / 10.3; pull 64x32x32 4.2 / 7.3, 96x48x32 5.9 / 9.0,
+// 128x48x32 9.3 / 10.1, 64^3 10.6 / 12.4, 128x64x64 17.3 / 17.7; FP16 AA 64x32x32 5.8 / 11.1, pull
+// 64x32x32 6.5 / 5.7, 64^3 14.0 / 8.2; D3Q27 FP32 tunnel 64x48x40 AA 12.7 / 10.8, pull 11.7 / 12.6.
+// A device that refuses the cooperative launch falls back to the graphs.
+static bool multi_fits(const lbm_s* h) {
+  const long long segments = (long long)(h->nxp / 32) * h->ny * h->nz;
+  const long long cap = (h->q == 19 ? 32ll : 16ll) * h->nsm;
+  if (h->prm.streaming != LBM_PULL) return segments <= cap;
+  return segments <= (kparams(h).split ? cap / 4 : 2 * cap);
+}
+
 constexpr int64_t MULTI_CHUNK = 4096;
 
 static bool steady_state(const lbm_s* h) {
@@ -955,7 +963,8 @@ static int64_t run_multi(lbm_handle h, int64_t n) {
 }
 
 static const char* const BROKEN_MSG =
-    "the handle is unusable: a learned-closure step gave up waiting for the tensor core twice";
+    "the handle is unusable: a learned-closure step gave up waiting for the tensor core twice, or a "
+    "multi-step launch for its blocks";
 
 lbm_status lbm_step(lbm_handle h, int64_t n) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
@@ -963,9 +972,7 @@ lbm_status lbm_step(lbm_handle h, int64_t n) {
   if (n < 0) return fail(h, LBM_EINVAL, "n must be >= 0");
   if (h->prm.closure == LBM_CLOSURE_MLP && !h->mlp_set)
     return fail(h, LBM_ESTATE, "MLP closure selected but lbm_set_closure was not called");
-  const long long multi_max = h->prm.streaming == LBM_PULL ? LBM_MULTI_MAX_CELLS : LBM_MULTI_MAX_CELLS_AA;
-  if (n >= 2 && !h->multi_off && h->prm.closure != LBM_CLOSURE_MLP &&
-      (long long)h->nxp * h->ny * h->nz <= multi_max) {
+  if (n >= 2 && !h->multi_off && h->prm.closure != LBM_CLOSURE_MLP && multi_fits(h)) {
     while (n > 0 && !steady_state(h)) {  // settle with single launches
       lbm_status s = run_steps(h, 1, 0);
       if (s != LBM_OK) return s;
@@ -1192,7 +1199,7 @@ lbm_status lbm_sync(lbm_handle h) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
   CUDA_TRY(h, cudaMemcpyAsync(h->status_host, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  if (*h->status_host & 4) {
+  if (*h->status_host & (4 | MULTI_GAVE_UP)) {
     h->broken = true;
     return fail(h, LBM_ECUDA, "%s", BROKEN_MSG);
   }
