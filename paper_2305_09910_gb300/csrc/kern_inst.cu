@@ -22,6 +22,16 @@ namespace lbm {
 #define LBM_LIST_FUSE_MAX (1ll << 18)
 #endif
 
+// The odd AA step of half storage, D3Q19: x-pairs or one cell per thread.  A pair warp with a lane
+// at an odd row end runs 3.4 times as long as a clean one, with an inflow, outflow or wall lane 6
+// times, and one cell per thread costs 1.22 times the clean pairs: pairs for rows of at least 11
+// pair warps per odd end and 23 per face.  FP16, us, pairs / one cell: 512x256x128 channel 282 /
+// 346, 256x130x121 91 / 98, 251x130x121 106 / 100, 375x190x187 tunnel 597 / 297.
+static bool odd_pairs(const KParams& p) {
+  const int faces = (p.face[0] != FACE_PERIODIC) + (p.face[1] != FACE_PERIODIC);
+  return (p.nxp + 63) / 64 >= 11 * (p.nx & 1) + 23 * faces;
+}
+
 template <int Q, class S, int LOAD, int STORE, bool STATS>
 static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll, int* nws) {
   if constexpr (Q == 19) {
@@ -45,7 +55,7 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
   // small FP16 lattices 69.5 -> 71.9 % of the copy bandwidth), a long one as k_step_list at its
   // own occupancy (the D3Q27 bluff body's 1.5 M listed cells: 74.6 % against 73.0 % in the pair
   // grid, whose 95 registers leave fewer warps for the latency-bound list).  The other D3Q27
-  // half steps take the one-cell kernel.
+  // pull steps (first after an import, statistics samples) take the one-cell kernel.
   if constexpr (sizeof(S) == 2 && (Q == 27 || LBM_SPLIT19) && LOAD == 2 && STORE == 2 && !STATS) {
     if (p.split && coll == 0) {
       dim3 g = L.grid;
@@ -64,14 +74,16 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       return;
     }
   }
-  // half storage, D3Q19: x-pairs, 64 x per warp
-  if constexpr (sizeof(S) == 2 && Q == 19) {
-    dim3 g = L.grid;
-    g.x = (p.nxp + 63) / 64;
-    if (nws) *nws = (int)g.x;
-    if (closure == CL_NONE) k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
-    else k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
-    return;
+  // half storage: x-pairs, 64 x per warp (D3Q27: the AA even step only, see above)
+  if (sizeof(S) == 2 && ((Q == 19 && (STORE != 1 || odd_pairs(p))) || STORE == 0)) {
+    if constexpr (sizeof(S) == 2 && (Q == 19 || STORE == 0)) {
+      dim3 g = L.grid;
+      g.x = (p.nxp + 63) / 64;
+      if (nws) *nws = (int)g.x;
+      if (closure == CL_NONE) k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
+      else k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
+      return;
+    }
   }
   if (nws) *nws = p.nxp / 32;
   if (closure == CL_NONE) k_step<Q, S, CL_NONE, LOAD, STORE, STATS><<<L.grid, L.block, 0, L.stream>>>(p);

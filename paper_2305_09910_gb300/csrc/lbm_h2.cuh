@@ -8,40 +8,18 @@
 // both cells at once in the packed FP32x2 pipe (float2 operands: FFMA2/FADD2/FMUL2); the two
 // results are rounded and packed into one word each.  This halves the memory instructions,
 // the address arithmetic and the arithmetic instructions per cell and doubles the bytes a
-// thread keeps in flight (LBM_H2_VEC=0 collides the two cells one after the other instead).
+// thread keeps in flight.
 //
-// Warps with any non-interior cell (boundary rules, periodic y/z wrap, skipped cells) take
-// the one-cell code for each of their two cells instead; the zero-gradient outflow passes
-// what cell x-1 receives from the lane that owns it (nx % 32 != 1 keeps x = nx-1 off lane 0).
+// In the pull step a lane with a cell that needs boundary rules, a periodic y/z wrap or no update
+// loads its two cells by the one-cell code, out of line; in the odd AA step a warp with such a lane
+// runs the one-cell code for its cells.  The zero-gradient outflow passes what cell x-1 receives
+// from the lane that owns it (nx % 32 != 1 keeps x = nx-1 off lane 0).
 // Block (32, 4) covers 64 x 4 cells of one z plane; grid (ceil(nxp/64), ceil(ny/4), nz).
 #pragma once
 
 #include "lbm_kernels.cuh"
 
 namespace lbm {
-
-template <class S> __device__ __forceinline__ float lo_of(uint32_t v);
-template <class S> __device__ __forceinline__ float hi_of(uint32_t v);
-template <> __device__ __forceinline__ float lo_of<__half>(uint32_t v) {
-  return __half2float(__ushort_as_half((unsigned short)(v & 0xffffu)));
-}
-template <> __device__ __forceinline__ float hi_of<__half>(uint32_t v) {
-  return __half2float(__ushort_as_half((unsigned short)(v >> 16)));
-}
-template <> __device__ __forceinline__ float lo_of<__nv_bfloat16>(uint32_t v) { return __uint_as_float(v << 16); }
-template <> __device__ __forceinline__ float hi_of<__nv_bfloat16>(uint32_t v) {
-  return __uint_as_float(v & 0xffff0000u);
-}
-
-template <class S> __device__ __forceinline__ uint32_t pack2(float a, float b);  // a in the low half
-template <> __device__ __forceinline__ uint32_t pack2<__half>(float a, float b) {
-  const __half2 h = __floats2half2_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-template <> __device__ __forceinline__ uint32_t pack2<__nv_bfloat16>(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 
 // 16-bit pattern of v rounded to the storage precision (round to nearest even)
 template <class S> __device__ __forceinline__ uint32_t bits16(float v);
@@ -126,17 +104,25 @@ __device__ __noinline__ void pair_fallback(const KParams& p, int x, int y, int z
 // step (out of line, below); the collision and the own-cell stores are common to all lanes, a
 // lane with a skipped (solid or padding) cell storing only its other cell's half.
 
-// Both cells of a boundary lane with the one-cell loads (load_state), packed into hs (the
-// loaded values are exact in the storage precision).  Out of line: the rule-by-rule loads are
+// Both cells of a boundary lane with the one-cell loads, packed into hs (the loaded values are
+// exact in the storage precision); ca, cb: class bytes.  Out of line: the rule-by-rule loads are
 // long, run for few lanes, and inlined they would crowd the instruction cache of every warp.
 template <int Q, class S, int PAR>
-__device__ __noinline__ void load_pair_rules(const KParams& p, int x, int y, int z, int cell, int clsA, int clsB,
+__device__ __noinline__ void load_pair_rules(const KParams& p, int x, int y, int z, int cell, int ca, int cb,
                                              uint32_t* hs, unsigned* oa, unsigned* ob) {
   float f[Q];
-  load_state<Q, S, PAR>(p, x, y, z, cell, clsA, f, *oa);
+  auto one = [&](int xc, int cc, int cbyte, unsigned& om) {
+    if (PAR != 0 && (cbyte & CLS_XFACE)) gather_xface<Q, S, PAR == 0 ? 1 : PAR>(p, xc, cc, f, om);
+    else load_state<Q, S, PAR, true>(p, xc, y, z, cc, cbyte & CLS_MASK, f, om);
+  };
+  unsigned om = 0;
+  one(x, cell, ca, om);
+  *oa = om;
 #pragma unroll
   for (int i = 0; i < Q; i++) hs[i] = bits16<S>(f[i]);
-  load_state<Q, S, PAR>(p, x + 1, y, z, cell + 1, clsB, f, *ob);
+  om = 0;
+  one(x + 1, cell + 1, cb, om);
+  *ob = om;
 #pragma unroll
   for (int i = 0; i < Q; i++) hs[i] |= bits16<S>(f[i]) << 16;
 }
@@ -224,6 +210,18 @@ __device__ __forceinline__ void pair_loads(const KParams& p, int x, int cell, ui
   }
 }
 
+// Statistics of the live cells of a pair.
+__device__ __forceinline__ void pair_stats(const Macro<float2>& M2, bool liveA, bool liveB, float (&v)[NSTAT]) {
+  float va[NSTAT], vb[NSTAT];
+  Macro<float> Ma, Mb;
+  Ma.ux = M2.ux.x; Ma.uy = M2.uy.x; Ma.uz = M2.uz.x;
+  Mb.ux = M2.ux.y; Mb.uy = M2.uy.y; Mb.uz = M2.uz.y;
+  stat_values(Ma, va);
+  stat_values(Mb, vb);
+#pragma unroll
+  for (int k = 0; k < NSTAT; k++) v[k] = (liveA ? va[k] : 0.f) + (liveB ? vb[k] : 0.f);
+}
+
 // early: the lane's pair is off the lattice faces and hpre holds its fast-path loads, issued
 // before the class load (in bounds whatever the classes).
 // The split step's inflow/outflow face cells (CLS_XFACE; their other sources are plain fluid
@@ -272,7 +270,7 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
     }
   } else {
     uint32_t hs[Q];
-    load_pair_rules<Q, S, LOAD>(p, x, y, z, cell, clsA, clsB, hs, &oa, &ob);
+    load_pair_rules<Q, S, LOAD>(p, x, y, z, cell, clsA | (xfA ? CLS_XFACE : 0), clsB | (xfB ? CLS_XFACE : 0), hs, &oa, &ob);
 #pragma unroll
     for (int i = 0; i < Q; i++) h[i] = hs[i];
   }
@@ -284,16 +282,7 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
   const bool liveB = SPLIT ? (clsB == CLS_INTERIOR || xfB) : clsB != CLS_SKIP;
   if ((liveA && !(rho.x > 0.f && rho.x < 3.0e38f)) || (liveB && !(rho.y > 0.f && rho.y < 3.0e38f)))
     flag_unstable(p);
-  if (STATS) {
-    float va[NSTAT], vb[NSTAT];
-    Macro<float> Ma, Mb;
-    Ma.ux = M2.ux.x; Ma.uy = M2.uy.x; Ma.uz = M2.uz.x;
-    Mb.ux = M2.ux.y; Mb.uy = M2.uy.y; Mb.uz = M2.uz.y;
-    stat_values(Ma, va);
-    stat_values(Mb, vb);
-#pragma unroll
-    for (int k = 0; k < NSTAT; k++) v[k] = (liveA ? va[k] : 0.f) + (liveB ? vb[k] : 0.f);
-  }
+  if (STATS) pair_stats(M2, liveA, liveB, v);
   if (liveA && liveB) {
 #pragma unroll
     for (int i = 0; i < Q; i++) st32(p, static_cast<S*>(p.fq[i]) + cell, h[i]);
@@ -306,14 +295,59 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
   }
 }
 
+// ---- AA even: every warp takes the pair path ----------------------------------------------
+// The even step reads and writes own slots whatever a cell's class: only the copied slots of the
+// outflow face (x = nx - 1) are taken from the upstream cell, and a lane with one cell that is not
+// updated stores its other half.  Before, one such lane (the odd end of a row, a wall, a seam)
+// sent its whole warp through the one-cell code twice: 251x130x121 FP16 D3Q19 channel 75 -> 66 us,
+// 375x190x187 tunnel 243 -> 206 us, 512x256x128 261 -> 244 us; D3Q27 (one-cell kernel before)
+// 102 -> 98, 342 -> 309 and 412 -> 367 us.
+template <int Q, class S, int CL, bool STATS>
+__device__ __forceinline__ void pair_even(const KParams& p, int x, int cell, int clsA, int clsB, float (&v)[NSTAT]) {
+  constexpr bool PACKED = Q == 27 ? LBM_H2_PACKED27 : LBM_H2_PACKED19;
+  const bool liveA = clsA != CLS_SKIP, liveB = clsB != CLS_SKIP;
+  uint32_t h[Q];
+  unsigned oa = 0, ob = 0;
+  if (liveA || liveB) {
+#pragma unroll
+    for (int i = 0; i < Q; i++) h[i] = ld32(p, plane_ptr<S>(p, i) + cell);
+    // after a streaming step the copied slots of the outflow face were not written
+    if (p.outflow && !p.nat_valid) {
+      const bool endA = x == p.nx - 1 && clsA == CLS_BOUNDARY, endB = x + 1 == p.nx - 1 && clsB == CLS_BOUNDARY;
+      if (endA || endB) {
+        const unsigned long long r = rule_at(p, cell + (endB ? 1 : 0));
+        unsigned m = 0;
+#pragma unroll
+        for (int i = 0; i < Q; i++)
+          if (cx(i) == -1 && ((r >> (2 * i)) & 3) == R_SPECIAL) m |= 1u << i;
+        (endB ? ob : oa) = m;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; i++) h[i] = 0;
+  }
+  outflow_fix_packed<Q>(p, 64 * blockIdx.x, h, oa, ob);
+  if (!liveA && !liveB) return;
+  Macro<float2> M2;
+  const float2 rho = collide_pair<Q, S, CL, PACKED>(p, h, STATS ? &M2 : nullptr);
+  if ((liveA && !(rho.x > 0.f && rho.x < 3.0e38f)) || (liveB && !(rho.y > 0.f && rho.y < 3.0e38f))) flag_unstable(p);
+  if (STATS) pair_stats(M2, liveA, liveB, v);
+  if (liveA && liveB) {
+#pragma unroll
+    for (int i = 0; i < Q; i++) st32(p, plane_ptr<S>(p, opp(i)) + cell, h[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; i++)
+      st16(p, plane_ptr<S>(p, opp(i)) + cell + (liveB ? 1 : 0), liveB ? h[i] >> 16 : h[i] & 0xffffu);
+  }
+}
+
 template <int Q, class S, int CL>
 __device__ __noinline__ void list_cell(const KParams& p, long long t);
 
-#ifndef LBM_H2_VEC
-#define LBM_H2_VEC 1
-#endif
 #ifndef LBM_H2_MINB
-#define LBM_H2_MINB (LBM_H2_VEC ? 7 : 8)
+#define LBM_H2_MINB 7
 #endif
 // STATS: also write the plane statistics of the state this step starts from (warp slot
 // blockIdx.x of each row, ceil(nxp/64) slots per row).
@@ -356,86 +390,39 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
   for (int k = 0; k < NSTAT; k++) v[k] = 0.f;
   if constexpr (STORE == 2) {
     pair_pull<Q, S, CL, LOAD, STATS, SPLIT>(p, x, y, z, cell, clsA, clsB, fast, v, early, hpre, xfA, xfB);
+  } else if constexpr (LOAD == 0) {
+    pair_even<Q, S, CL, STATS>(p, x, cell, clsA, clsB, v);
   } else if (__all_sync(0xffffffffu, fast)) {
+    // AA odd, all lanes interior: gather, and store back into the slots the gather read
     uint32_t h[Q];
 #pragma unroll
     for (int i = 0; i < Q; i++) {
-      if (LOAD == 0) {
-        h[i] = ld32(p, plane_ptr<S>(p, i) + cell);
+      const S* base = static_cast<const S*>(p.ga[i]);
+      if (cx(i) == 0) {
+        h[i] = ld32(p, base + cell);
       } else {
-        const S* base = static_cast<const S*>(LOAD == 2 ? p.gb[i] : p.ga[i]);
-        if (cx(i) == 0) {
-          h[i] = ld32(p, base + cell);
-        } else {
-          int a, b;
-          xsrc(cx(i), p, x, cell, a, b);
-          const uint32_t lo = ld16(p, base + a);
-          const uint32_t hi = ld16(p, base + b);
-          h[i] = lo | (hi << 16);
-        }
+        int a, b;
+        xsrc(cx(i), p, x, cell, a, b);
+        const uint32_t lo = ld16(p, base + a);
+        const uint32_t hi = ld16(p, base + b);
+        h[i] = lo | (hi << 16);
       }
     }
-#if LBM_H2_VEC
-    // both cells at once in the packed FP32x2 pipe
-    float2 f[Q];
-#pragma unroll
-    for (int i = 0; i < Q; i++) f[i] = make_float2(lo_of<S>(h[i]), hi_of<S>(h[i]));
     Macro<float2> M2;
-    const float2 rho = collide<Q, CL, float2, false>(p, f, STATS ? &M2 : nullptr);
-    if (STATS) {
-      float va[NSTAT], vb[NSTAT];
-      Macro<float> Ma, Mb;
-      Ma.ux = M2.ux.x; Ma.uy = M2.uy.x; Ma.uz = M2.uz.x;
-      Mb.ux = M2.ux.y; Mb.uy = M2.uy.y; Mb.uz = M2.uz.y;
-      stat_values(Ma, va);
-      stat_values(Mb, vb);
+    const float2 rho = collide_pair<Q, S, CL, false>(p, h, STATS ? &M2 : nullptr);
+    if (STATS) pair_stats(M2, true, true, v);
+    if (!(rho.x > 0.f && rho.x < 3.0e38f) || !(rho.y > 0.f && rho.y < 3.0e38f)) flag_unstable(p);
 #pragma unroll
-      for (int k = 0; k < NSTAT; k++) v[k] = va[k] + vb[k];
-    }
-#pragma unroll
-    for (int i = 0; i < Q; i++) h[i] = pack2<S>(f[i].x, f[i].y);
-    const float ra = rho.x, rb = rho.y;
-#else
-    // first cell: unpack, collide, round back into the low halves
-    float f[Q];
-    Macro<float> Ma, Mb;
-#pragma unroll
-    for (int i = 0; i < Q; i++) f[i] = lo_of<S>(h[i]);
-    const float ra = collide<Q, CL, float, false>(p, f, STATS ? &Ma : nullptr);
-#pragma unroll
-    for (int i = 0; i < Q; i++) h[i] = __byte_perm(h[i], bits16<S>(f[i]), 0x3254);
-    // second cell: the high halves
-#pragma unroll
-    for (int i = 0; i < Q; i++) f[i] = hi_of<S>(h[i]);
-    const float rb = collide<Q, CL, float, false>(p, f, STATS ? &Mb : nullptr);
-    if (STATS) {
-      float va[NSTAT], vb[NSTAT];
-      stat_values(Ma, va);
-      stat_values(Mb, vb);
-#pragma unroll
-      for (int k = 0; k < NSTAT; k++) v[k] = va[k] + vb[k];
-    }
-#pragma unroll
-    for (int i = 0; i < Q; i++) h[i] = __byte_perm(h[i], bits16<S>(f[i]), 0x5410);
-#endif
-    if (!(ra > 0.f && ra < 3.0e38f) || !(rb > 0.f && rb < 3.0e38f)) flag_unstable(p);
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      if (STORE == 0) {
-        st32(p, plane_ptr<S>(p, opp(i)) + cell, h[i]);
-      } else if (STORE == 2) {
-        st32(p, static_cast<S*>(p.fq[i]) + cell, h[i]);
-      } else {  // back into the slots the gather of direction i read: f*_opp(i)
-        S* base = static_cast<S*>(p.ga[i]);
-        const uint32_t w = h[opp(i)];
-        if (cx(i) == 0) {
-          st32(p, base + cell, w);
-        } else {
-          int a, b;
-          xsrc(cx(i), p, x, cell, a, b);
-          st16(p, base + a, w & 0xffffu);
-          st16(p, base + b, w >> 16);
-        }
+    for (int i = 0; i < Q; i++) {  // the slots of direction i take f*_opp(i)
+      S* base = static_cast<S*>(p.ga[i]);
+      const uint32_t w = h[opp(i)];
+      if (cx(i) == 0) {
+        st32(p, base + cell, w);
+      } else {
+        int a, b;
+        xsrc(cx(i), p, x, cell, a, b);
+        st16(p, base + a, w & 0xffffu);
+        st16(p, base + b, w >> 16);
       }
     }
   } else {
