@@ -37,15 +37,15 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
   if constexpr (Q == 19) {
     if (coll == 1) {
       if (nws) *nws = p.nxp / 32;
-      if (closure == CL_NONE) k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 1><<<L.grid, L.block, 0, L.stream>>>(p);
-      else k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 1><<<L.grid, L.block, 0, L.stream>>>(p);
+      if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 1>, L.grid, L.block, L.stream, p);
+      else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 1>, L.grid, L.block, L.stream, p);
       return;
     }
   }
   if (coll == 2) {  // regularised collision: one cell per thread, every stencil and storage
     if (nws) *nws = p.nxp / 32;
-    if (closure == CL_NONE) k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 2><<<L.grid, L.block, 0, L.stream>>>(p);
-    else k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 2><<<L.grid, L.block, 0, L.stream>>>(p);
+    if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 2>, L.grid, L.block, L.stream, p);
+    else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 2>, L.grid, L.block, L.stream, p);
     return;
   }
   // half storage, gather step of two-grid pull without statistics (both stencils; D3Q19 unless
@@ -64,12 +64,12 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       const long long extra = (p.nblist + per - 1) / per;
       const bool fused = p.nblist <= LBM_LIST_FUSE_MAX && g.z + extra <= 65535;
       if (fused) g.z += (unsigned)extra;
-      if (closure == CL_NONE) k_step_h2<Q, S, CL_NONE, 2, 2, false, true><<<g, L.block, 0, L.stream>>>(p);
-      else k_step_h2<Q, S, CL_SMAG, 2, 2, false, true><<<g, L.block, 0, L.stream>>>(p);
+      if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true>, g, L.block, L.stream, p);
+      else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true>, g, L.block, L.stream, p);
       if (!fused) {
         const unsigned nb = (unsigned)((p.nblist + 127) / 128);
-        if (closure == CL_NONE) k_step_list<Q, S, CL_NONE><<<nb, 128, 0, L.stream>>>(p);
-        else k_step_list<Q, S, CL_SMAG><<<nb, 128, 0, L.stream>>>(p);
+        if (closure == CL_NONE) launch_chained(k_step_list<Q, S, CL_NONE>, nb, 128, L.stream, p);
+        else launch_chained(k_step_list<Q, S, CL_SMAG>, nb, 128, L.stream, p);
       }
       return;
     }
@@ -80,14 +80,14 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       dim3 g = L.grid;
       g.x = (p.nxp + 63) / 64;
       if (nws) *nws = (int)g.x;
-      if (closure == CL_NONE) k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
-      else k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS><<<g, L.block, 0, L.stream>>>(p);
+      if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS>, g, L.block, L.stream, p);
+      else launch_chained(k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS>, g, L.block, L.stream, p);
       return;
     }
   }
   if (nws) *nws = p.nxp / 32;
-  if (closure == CL_NONE) k_step<Q, S, CL_NONE, LOAD, STORE, STATS><<<L.grid, L.block, 0, L.stream>>>(p);
-  else k_step<Q, S, CL_SMAG, LOAD, STORE, STATS><<<L.grid, L.block, 0, L.stream>>>(p);
+  if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS>, L.grid, L.block, L.stream, p);
+  else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS>, L.grid, L.block, L.stream, p);
 }
 
 template <int Q, class S, int LOAD, int STORE>

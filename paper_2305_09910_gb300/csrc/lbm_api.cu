@@ -397,6 +397,7 @@ __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >
 template <class E>
 __global__ void __launch_bounds__(256) k_refine_explode(RefPlanes rp, int nd, int nxf, int nyf, int nxpf,
                                                         int nxpc, int s) {
+  chain_begin();
   const long long plane = (long long)nyf * nxf;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nd * plane;
        t += (long long)gridDim.x * blockDim.x) {
@@ -412,6 +413,7 @@ __global__ void __launch_bounds__(256) k_refine_explode(RefPlanes rp, int nd, in
 template <class S>
 __global__ void __launch_bounds__(256) k_refine_coalesce(RefPlanes rp, int nd, int nxc, int nyc, int nxpc,
                                                          int nxpf) {
+  chain_begin();
   const long long plane = (long long)nyc * nxc;
   const int nxf = 2 * nxc, nyf = 2 * nyc;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nd * plane;
@@ -1159,9 +1161,9 @@ lbm_status lbm_refine_explode(lbm_handle coarse, int coarse_face, lbm_handle fin
   const long long n = (long long)nd * fine->nx * fine->ny;
   const int blocks = (int)std::min<long long>((n + 255) / 256, (long long)fine->nsm * 8);
   if (fine->prm.precision == LBM_F32)
-    k_refine_explode<uint32_t><<<blocks, 256, 0, fine->stream>>>(rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
+    launch_chained(k_refine_explode<uint32_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
   else
-    k_refine_explode<uint16_t><<<blocks, 256, 0, fine->stream>>>(rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
+    launch_chained(k_refine_explode<uint16_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
   CUDA_TRY(fine, cudaGetLastError());
   return stream_join(fine, coarse, fine);
 }
@@ -1181,14 +1183,13 @@ lbm_status lbm_refine_coalesce(lbm_handle fine, int fine_face, lbm_handle coarse
   const int blocks = (int)std::min<long long>((n + 255) / 256, (long long)coarse->nsm * 8);
   switch (coarse->prm.precision) {
     case LBM_F32:
-      k_refine_coalesce<float><<<blocks, 256, 0, coarse->stream>>>(rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
+      launch_chained(k_refine_coalesce<float>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
     case LBM_F16_SHIFTED:
-      k_refine_coalesce<__half><<<blocks, 256, 0, coarse->stream>>>(rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
+      launch_chained(k_refine_coalesce<__half>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
     default:
-      k_refine_coalesce<__nv_bfloat16><<<blocks, 256, 0, coarse->stream>>>(rp, nd, coarse->nx, coarse->ny, coarse->nxp,
-                                                                          fine->nxp);
+      launch_chained(k_refine_coalesce<__nv_bfloat16>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
   }
   CUDA_TRY(coarse, cudaGetLastError());

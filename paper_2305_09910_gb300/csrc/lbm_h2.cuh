@@ -354,6 +354,7 @@ __device__ __noinline__ void list_cell(const KParams& p, long long t);
 template <int Q, class S, int CL, int LOAD, int STORE, bool STATS = false, bool SPLIT = false>
 __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_step_h2(const __grid_constant__ KParams p) {
   static_assert(sizeof(S) == 2, "two 16-bit populations per word");
+  chain_begin();
   if constexpr (SPLIT) {
     // blocks past the last z plane take the listed cells, 128 per block: they follow the pair
     // blocks in launch order and fill the SMs the pair grid's tail leaves idle
@@ -506,6 +507,7 @@ __device__ __noinline__ void list_cell(const KParams& p, long long t) {
 // blocks to follow the x-pair grid in its z dimension.
 template <int Q, class S, int CL>
 __global__ void __launch_bounds__(128) k_step_list(const __grid_constant__ KParams p) {
+  chain_begin();
   list_cell<Q, S, CL>(p, blockIdx.x * 128ll + threadIdx.x);
 }
 

@@ -13,6 +13,21 @@ struct Launch {
   cudaStream_t stream;
 };
 
+// Launch of a kernel that begins with chain_begin().
+template <class... P, class... A>
+inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t stream, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // (the callers read cudaGetLastError)
+}
+
 template <int Q, class S>
 cudaError_t launch_step(const KParams& p, int closure, int parity, const Launch& L, bool stats = false,
                         int* nws = nullptr, int coll = 0);
