@@ -199,7 +199,17 @@ template <int Q, class S, int PAR>
 static void export_par(const KParams& p, int mode, const ExportArgs& a, const Launch& L) {
   switch (mode) {
     case EX_POP: k_export<Q, S, PAR, EX_POP><<<L.grid, L.block, 0, L.stream>>>(p, a); break;
-    case EX_MOM: k_export<Q, S, PAR, EX_MOM><<<L.grid, L.block, 0, L.stream>>>(p, a); break;
+    case EX_MOM:
+      // half storage: two cells per thread (64-bit stores need even rows and 8-byte aligned arrays),
+      // D3Q27 in natural layout only: gathered, its 80 registers cost more than the pairs give
+      // (FP16 512x256x128 AA after an even step 253 -> 179 us, pull 283 us against 303)
+      if constexpr (sizeof(S) == 2 && (Q == 19 || PAR == 0)) {
+        const int vec = p.nx % 2 == 0 && (uintptr_t)a.rho % 8 == 0 && (uintptr_t)a.u % 8 == 0;
+        k_moments_h2<Q, S, PAR><<<dim3((p.nxp + 63) / 64, L.grid.y, L.grid.z), L.block, 0, L.stream>>>(p, a, vec);
+      } else {
+        k_export<Q, S, PAR, EX_MOM><<<L.grid, L.block, 0, L.stream>>>(p, a);
+      }
+      break;
     case EX_SUM: {
       const int rows = p.ny * p.nz, cnt = (rows + LBM_ROW_BLOCKS - 1) / LBM_ROW_BLOCKS;
       const int nblk = (rows + cnt - 1) / cnt;

@@ -185,6 +185,22 @@ __device__ __forceinline__ float2 collide_pair(const KParams& p, uint32_t (&h)[Q
   }
 }
 
+// Natural layout after a streaming step: the copied slots of the outflow face were not written;
+// their directions in the cell at x = nx - 1 (oa: the lane's first cell, ob: its second).
+template <int Q>
+__device__ __forceinline__ void own_outflow_masks(const KParams& p, int x, int cell, int clsA, int clsB, unsigned& oa,
+                                                  unsigned& ob) {
+  if (!p.outflow || p.nat_valid) return;
+  const bool endA = x == p.nx - 1 && clsA == CLS_BOUNDARY, endB = x + 1 == p.nx - 1 && clsB == CLS_BOUNDARY;
+  if (!endA && !endB) return;
+  const unsigned long long r = rule_at(p, cell + (endB ? 1 : 0));
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < Q; i++)
+    if (cx(i) == -1 && ((r >> (2 * i)) & 3) == R_SPECIAL) m |= 1u << i;
+  (endB ? ob : oa) = m;
+}
+
 // SPLIT (gather step of a handle with a cell list, no statistics): only the interior cells and
 // the simple inflow/outflow face cells are updated here, the listed ones by k_step_list.  A lane with one interior cell loads both cells'
 // words (the other cell's sources, one x further, stay inside the arrays) and stores one half.
@@ -196,7 +212,7 @@ __device__ __forceinline__ void pair_loads(const KParams& p, int x, int cell, ui
     if (LOAD == 0) {
       h[i] = ld32(p, plane_ptr<S>(p, i) + cell);
     } else {
-      const S* base = static_cast<const S*>(p.gb[i]);
+      const S* base = static_cast<const S*>(LOAD == 1 ? p.ga[i] : p.gb[i]);
       if (cx(i) == 0) {
         h[i] = chk(p, base + cell, 4, CHK_POP) ? ldh_u32(base + cell) : 0u;
       } else {
@@ -311,18 +327,7 @@ __device__ __forceinline__ void pair_even(const KParams& p, int x, int cell, int
   if (liveA || liveB) {
 #pragma unroll
     for (int i = 0; i < Q; i++) h[i] = ld32(p, plane_ptr<S>(p, i) + cell);
-    // after a streaming step the copied slots of the outflow face were not written
-    if (p.outflow && !p.nat_valid) {
-      const bool endA = x == p.nx - 1 && clsA == CLS_BOUNDARY, endB = x + 1 == p.nx - 1 && clsB == CLS_BOUNDARY;
-      if (endA || endB) {
-        const unsigned long long r = rule_at(p, cell + (endB ? 1 : 0));
-        unsigned m = 0;
-#pragma unroll
-        for (int i = 0; i < Q; i++)
-          if (cx(i) == -1 && ((r >> (2 * i)) & 3) == R_SPECIAL) m |= 1u << i;
-        (endB ? ob : oa) = m;
-      }
-    }
+    own_outflow_masks<Q>(p, x, cell, clsA, clsB, oa, ob);
   } else {
 #pragma unroll
     for (int i = 0; i < Q; i++) h[i] = 0;
@@ -430,6 +435,68 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
     pair_fallback<Q, S, CL, LOAD, STORE, STATS>(p, x, y, z, cell, clsA, clsB, v);
   }
   if (STATS) stat_warp_store(p, y, z, blockIdx.x, (p.nxp + 63) / 64, v);
+}
+
+// ---- fields of the current state, half storage -----------------------------------------------
+// rho and u of two x-adjacent cells per thread (the one-cell export's values): packed loads, both
+// cells' sums in the FP32x2 pipe, 64-bit stores where the arrays and rows allow them (vec).
+// Bound by HBM and latency; one cell per thread moved 64 bytes per load
+// and warp.  1024x512x512 D3Q19 FP16 pull 3513 -> 2660 us, 375x190x187 FP16 AA tunnel 157 -> 121 us.
+template <int Q, class S, int PAR>
+__global__ void __launch_bounds__(128, Q == 27 ? 6 : 8) k_moments_h2(const __grid_constant__ KParams p, ExportArgs a, int vec) {
+  const int x = 2 * (blockIdx.x * 32 + threadIdx.x);
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  const int z = blockIdx.z;
+  if (y >= p.ny) return;  // whole warp
+  const int cell = cidx(p, x, y, z);
+  uint32_t h[Q];
+#pragma unroll
+  for (int i = 0; i < Q; i++) h[i] = 0;
+  // own slots of any cell, or the gather of a pair off the faces: in bounds whatever the classes, so
+  // in flight with the class load below
+  const bool early = PAR == 0 ? x < p.nx
+                              : x >= 1 && x + 1 < p.nx - 1 && y >= 1 && y < p.ny - 1 && z >= 1 && z < p.nz - 1;
+  if (early) pair_loads<Q, S, PAR>(p, x, cell, h);
+  int ca = CLS_SKIP, cb = CLS_SKIP;
+  if (x < p.nx) {
+    const unsigned c2 = chk(p, p.cls + cell, 2, CHK_CLS) ? *reinterpret_cast<const unsigned short*>(p.cls + cell) : 0x0202u;
+    ca = c2 & 0xff;
+    cb = x + 1 < p.nx ? (int)(c2 >> 8) : CLS_SKIP;
+  }
+  const bool liveA = (ca & CLS_MASK) != CLS_SKIP, liveB = (cb & CLS_MASK) != CLS_SKIP;
+  unsigned oa = 0, ob = 0;
+  if (PAR == 0) {
+    own_outflow_masks<Q>(p, x, cell, ca & CLS_MASK, cb & CLS_MASK, oa, ob);
+  } else if ((ca & CLS_MASK) == CLS_INTERIOR && (cb & CLS_MASK) == CLS_INTERIOR) {
+    if (!early) pair_loads<Q, S, PAR>(p, x, cell, h);
+  } else if (liveA || liveB) {
+    uint32_t hs[Q];
+    load_pair_rules<Q, S, PAR>(p, x, y, z, cell, ca, cb, hs, &oa, &ob);
+#pragma unroll
+    for (int i = 0; i < Q; i++) h[i] = hs[i];
+  }
+  outflow_fix_packed<Q>(p, 64 * blockIdx.x, h, oa, ob);
+  if (x >= p.nx) return;
+  PackedPops<Q, S> pops{h};
+  const Macro<float2> M = macro_acc<Q, false, float2>(p, pops);
+  const long long dense = ((long long)z * p.ny + y) * p.nx + x;
+  const long long N = (long long)p.nx * p.ny * p.nz;
+  auto put = [&](float* out, float2 v) {
+    v.x = liveA ? v.x : 0.f;
+    v.y = liveB ? v.y : 0.f;
+    if (vec) {
+      *reinterpret_cast<float2*>(out + dense) = v;
+    } else {
+      out[dense] = v.x;
+      if (x + 1 < p.nx) out[dense + 1] = v.y;
+    }
+  };
+  if (a.rho) put(a.rho, M.rho);
+  if (a.u) {
+    put(a.u, M.ux);
+    put(a.u + N, M.uy);
+    put(a.u + 2 * N, M.uz);
+  }
 }
 
 // ---- the listed cells of a split pull step ---------------------------------------------------
