@@ -152,12 +152,6 @@ __device__ __forceinline__ void outflow_fix_packed(const KParams& p, int x0, uin
 #ifndef LBM_H2_MINB27
 #define LBM_H2_MINB27 5
 #endif
-#ifndef LBM_H2_EARLY19
-#define LBM_H2_EARLY19 0
-#endif
-#ifndef LBM_H2_EARLY27
-#define LBM_H2_EARLY27 1
-#endif
 
 // The collision of both cells (float2 lanes).  PACKED: the populations stay packed and are
 // unpacked at each use (fewer live registers); else they are unpacked once into float2 values.
@@ -238,8 +232,6 @@ __device__ __forceinline__ void pair_stats(const Macro<float2>& M2, bool liveA, 
   for (int k = 0; k < NSTAT; k++) v[k] = (liveA ? va[k] : 0.f) + (liveB ? vb[k] : 0.f);
 }
 
-// early: the lane's pair is off the lattice faces and hpre holds its fast-path loads, issued
-// before the class load (in bounds whatever the classes).
 // The split step's inflow/outflow face cells (CLS_XFACE; their other sources are plain fluid
 // neighbours, so the fast loads hold them): the directions crossing the face take the
 // moving-wall value of the own cell (inflow, x = 0: always the lane's first cell) or what the
@@ -268,8 +260,7 @@ __device__ __forceinline__ void xface_fix(const KParams& p, int x, int cell, boo
 
 template <int Q, class S, int CL, int LOAD, bool STATS, bool SPLIT>
 __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z, int cell, int clsA, int clsB,
-                                          bool fast, float (&v)[NSTAT], bool early, const uint32_t (&hpre)[Q],
-                                          bool xfA, bool xfB) {
+                                          bool fast, float (&v)[NSTAT], bool xfA, bool xfB) {
   constexpr bool PACKED = Q == 27 ? LBM_H2_PACKED27 : LBM_H2_PACKED19;
   static_assert(!SPLIT || (LOAD == 2 && !STATS), "the split runs the gather step without statistics");
   uint32_t h[Q];
@@ -279,11 +270,7 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
     fast = true;
   }
   if (fast) {
-    if (!early) pair_loads<Q, S, LOAD>(p, x, cell, h);
-    else {
-#pragma unroll
-      for (int i = 0; i < Q; i++) h[i] = hpre[i];
-    }
+    pair_loads<Q, S, LOAD>(p, x, cell, h);
   } else {
     uint32_t hs[Q];
     load_pair_rules<Q, S, LOAD>(p, x, y, z, cell, clsA | (xfA ? CLS_XFACE : 0), clsB | (xfB ? CLS_XFACE : 0), hs, &oa, &ob);
@@ -374,13 +361,8 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
   const int z = blockIdx.z;
   if (y >= p.ny) return;  // whole warp
   const int cell = cidx(p, x, y, z);
-  // two-grid pull, lanes off the lattice faces: the fast-path loads go out with the class load
-  // (D3Q27 split step; for D3Q19 pairs measured slower, 60.4k against 64.7k MLUPS)
-  constexpr bool EARLY = Q == 27 ? LBM_H2_EARLY27 : LBM_H2_EARLY19;
-  const bool early = EARLY && STORE == 2 && LOAD == 2 && x >= 1 && x + 1 < p.nx - 1 && y >= 1 && y < p.ny - 1 &&
-                     z >= 1 && z < p.nz - 1;
-  uint32_t hpre[Q];
-  if (early) pair_loads<Q, S, LOAD>(p, x, cell, hpre);
+  // (the gather issued with the class load instead of after it: D3Q19 FP16 channel 501 -> 506 us,
+  // D3Q27 FP16 tunnel 2466 -> 2488 us)
   int ca_ = CLS_SKIP, cb_ = CLS_SKIP;
   if (x < p.nx) {
     const unsigned c2 = chk(p, p.cls + cell, 2, CHK_CLS) ? *reinterpret_cast<const unsigned short*>(p.cls + cell) : 0x0202u;
@@ -395,7 +377,7 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
 #pragma unroll
   for (int k = 0; k < NSTAT; k++) v[k] = 0.f;
   if constexpr (STORE == 2) {
-    pair_pull<Q, S, CL, LOAD, STATS, SPLIT>(p, x, y, z, cell, clsA, clsB, fast, v, early, hpre, xfA, xfB);
+    pair_pull<Q, S, CL, LOAD, STATS, SPLIT>(p, x, y, z, cell, clsA, clsB, fast, v, xfA, xfB);
   } else if constexpr (LOAD == 0) {
     pair_even<Q, S, CL, STATS>(p, x, cell, clsA, clsB, v);
   } else if (__all_sync(0xffffffffu, fast)) {
