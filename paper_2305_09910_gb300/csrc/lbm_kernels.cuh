@@ -1178,10 +1178,79 @@ __device__ __forceinline__ void relax_reg(const KParams& p, float (&f)[Q], const
 //   j: rho u, F;  q: -2/3 rho u, -2/3 F;  3p_xx: rho (3u_x^2 - u^2), 6 u_x F_x - 2 u.F;
 //   3pi_xx: -1/2 of 3p_xx (both);  p_ww: rho (u_y^2 - u_z^2), 2 (u_y F_y - u_z F_z);
 //   pi_ww: -1/2 of p_ww;  p_ab: rho u_a u_b, u_a F_b + u_b F_a;  m: 0, 0.
+// Both transforms go by shells of the pair sums s and differences a (|c|^2 = 1 along x, y, z and
+// |c|^2 = 2 in the planes xy, xz, yz): every row is a combination of few shell sums, e.g. 3p_xx =
+// A + B and 3pi_xx = -2 A + B with A = 2 s_x - s_y - s_z, B = s_xy + s_xz - 2 s_yz.  About 45
+// operations each way; row by row they took 110 each.  512x256x256 FP32 pull, with one more
+// resident block for it, 868 -> 813 us.
+// Half storage keeps the row-by-row form: another rounding in float32 flips roundings of the stored
+// values, and after some tens of steps the flow differs by the storage rounding noise itself.
+__device__ __forceinline__ void mrt_shell_moments(float f0, const float (&sp)[9], const float (&ap)[9], float (&m)[19]) {
+  const float syz1 = vadd(sp[1], sp[2]), S1 = vadd(sp[0], syz1);
+  const float sxy = vadd(sp[3], sp[4]), sxz = vadd(sp[5], sp[6]), syz = vadd(sp[7], sp[8]);
+  const float sxx = vadd(sxy, sxz), S2 = vadd(sxx, syz);
+  m[0] = vadd(f0, vadd(S1, S2));
+  m[1] = vfma(-30.f, f0, vfma(-11.f, S1, vmul(8.f, S2)));
+  m[2] = vfma(12.f, f0, vfma(-4.f, S1, S2));
+  const float A = vfma(2.f, sp[0], -syz1), B = vfma(-2.f, syz, sxx);
+  const float C = vsub(sp[1], sp[2]), D = vsub(sxy, sxz);
+  m[9] = vadd(A, B);
+  m[10] = vfma(-2.f, A, B);
+  m[11] = vadd(C, D);
+  m[12] = vfma(-2.f, C, D);
+  m[13] = vsub(sp[3], sp[4]);
+  m[14] = vsub(sp[7], sp[8]);
+  m[15] = vsub(sp[5], sp[6]);
+  const float xy = vadd(ap[3], ap[4]), yx = vsub(ap[3], ap[4]);  // x and y parts of the xy shell
+  const float xz = vadd(ap[5], ap[6]), zx = vsub(ap[5], ap[6]);
+  const float yz = vadd(ap[7], ap[8]), zy = vsub(ap[7], ap[8]);
+  const float X2 = vadd(xy, xz), Y2 = vadd(yx, yz), Z2 = vadd(zx, zy);
+  m[3] = vadd(ap[0], X2);
+  m[4] = vfma(-4.f, ap[0], X2);
+  m[5] = vadd(ap[1], Y2);
+  m[6] = vfma(-4.f, ap[1], Y2);
+  m[7] = vadd(ap[2], Z2);
+  m[8] = vfma(-4.f, ap[2], Z2);
+  m[16] = vsub(xy, xz);
+  m[17] = vsub(yz, yx);
+  m[18] = vsub(zx, zy);
+}
+
+__device__ __forceinline__ void mrt_shell_back(float (&f)[19], const float (&m)[19]) {
+  f[0] = vadd(f[0], vfma(-30.f, m[1], vfma(12.f, m[2], m[0])));
+  auto back = [&](auto I_, float e, float o) {  // even part e, odd part o of a pair's update
+    constexpr int I = decltype(I_)::value;
+    constexpr int PP = prim(I), R = PP == I ? I + 1 : I;
+    f[PP] = vadd(f[PP], vadd(e, o));
+    f[R] = vadd(f[R], vsub(e, o));
+  };
+  {
+    const float b1 = vfma(-11.f, m[1], vfma(-4.f, m[2], m[0])), b2 = vfma(8.f, m[1], vadd(m[0], m[2]));
+    const float u = vfma(-2.f, m[10], m[9]), v = vfma(-2.f, m[12], m[11]);
+    const float bu = vsub(b1, u);
+    back(std::integral_constant<int, 1>{}, vfma(2.f, u, b1), vfma(-4.f, m[4], m[3]));
+    back(std::integral_constant<int, 3>{}, vadd(bu, v), vfma(-4.f, m[6], m[5]));
+    back(std::integral_constant<int, 5>{}, vsub(bu, v), vfma(-4.f, m[8], m[7]));
+    const float w = vadd(m[9], m[10]), q = vadd(m[11], m[12]), bw = vadd(b2, w);
+    const float exy = vadd(bw, q), exz = vsub(bw, q), eyz = vfma(-2.f, w, b2);
+    const float X = vadd(m[3], m[4]), Y = vadd(m[5], m[6]), Z = vadd(m[7], m[8]);
+    const float xp = vadd(X, m[16]), xm = vsub(X, m[16]);  // X in the xy, xz shells
+    const float yp = vadd(Y, m[17]), ym = vsub(Y, m[17]);  // Y in the yz, xy shells
+    const float zp = vadd(Z, m[18]), zm = vsub(Z, m[18]);  // Z in the xz, yz shells
+    back(std::integral_constant<int, 7>{}, vadd(exy, m[13]), vadd(xp, ym));
+    back(std::integral_constant<int, 9>{}, vsub(exy, m[13]), vsub(xp, ym));
+    back(std::integral_constant<int, 11>{}, vadd(exz, m[15]), vadd(xm, zp));
+    back(std::integral_constant<int, 13>{}, vsub(exz, m[15]), vsub(xm, zp));
+    back(std::integral_constant<int, 15>{}, vadd(eyz, m[14]), vadd(yp, zm));
+    back(std::integral_constant<int, 17>{}, vsub(eyz, m[14]), vsub(yp, zm));
+  }
+}
+
+template <bool SHELL>
 __device__ __forceinline__ void relax_mrt(const KParams& p, float (&f)[19], const Macro<float>& M, float wnu) {
+  // pair sums and differences in the primary orientation: x, y, z, then ++ and +- of xy, xz, yz
   float sp[9], ap[9];
   {
-    // pair sums in the primary orientation
     auto fill = [&](auto I_) {
       constexpr int I = decltype(I_)::value;
       constexpr int PP = prim(I), R = PP == I ? I + 1 : I;
@@ -1199,7 +1268,8 @@ __device__ __forceinline__ void relax_mrt(const KParams& p, float (&f)[19], cons
     fill(std::integral_constant<int, 17>{});
   }
   float m[19];
-  mrt_pair_moments(f[0], sp, ap, m, std::make_integer_sequence<int, 19>{});
+  if constexpr (SHELL) mrt_shell_moments(f[0], sp, ap, m);
+  else mrt_pair_moments(f[0], sp, ap, m, std::make_integer_sequence<int, 19>{});
   const float ux = M.ux, uy = M.uy, uz = M.uz, rho = M.rho;
   const float Fx = p.F[0], Fy = p.F[1], Fz = p.F[2];
   const float u2 = vfma(uz, uz, vfma(uy, uy, vmul(ux, ux)));
@@ -1234,14 +1304,16 @@ __device__ __forceinline__ void relax_mrt(const KParams& p, float (&f)[19], cons
     // (the momentum rows of df lack the half force of j: m_j(df) - j = -F/2)
     m[k] = vmul(vfma(-s, vsub(m[k], meq[k]), vmul(vfma(s, -0.5f, 1.f), mf[k])), 1.f / (float)mrt_norm(k));
   }
-  {
+  if constexpr (SHELL) {
+    mrt_shell_back(f, m);
+  } else {
     float e0 = 0.f;
 #pragma unroll
     for (int k = 0; k < 19; k++)
       if (mrt_even(k) && mrt_row(k, 0) != 0) e0 = vfma(m[k], (float)mrt_row(k, 0), e0);
     f[0] = vadd(f[0], e0);
+    mrt_pairs_back(f, m, std::make_integer_sequence<int, 9>{});
   }
-  mrt_pairs_back(f, m, std::make_integer_sequence<int, 9>{});
 }
 
 // Stream-collide arithmetic of one cell (or two) without a learned closure: plain TRT or
@@ -1265,7 +1337,7 @@ __device__ __forceinline__ V collide(const KParams& p, V (&f)[Q], Macro<V>* mout
   }
   if constexpr (COLL == 1) {
     static_assert(Q == 19 && std::is_same<V, float>::value, "MRT: D3Q19, one cell per thread");
-    relax_mrt(p, f, M, wp);
+    relax_mrt<ACC>(p, f, M, wp);
   } else if constexpr (COLL == 2) {
     static_assert(std::is_same<V, float>::value, "regularised: one cell per thread");
     relax_reg<Q>(p, f, M, wp);
@@ -1400,7 +1472,8 @@ static __global__ void __launch_bounds__(256) k_stats_total(const float* stats_w
 // Resident blocks per SM the step is compiled for (registers per thread = 65536 / (128 x
 // this)): more resident warps keep more loads in flight.  D3Q19 TRT and regularised: 10 (48
 // registers; the pull step spills nothing and measured 10 % faster than at 8); D3Q27: 9 (56
-// registers, no spill; pull 5 % faster); MRT: 8, above which it spills.
+// registers, no spill; pull 5 % faster); MRT: FP32 storage 9, in the AA odd step 8 (it
+// spills at 9: 906 against 875 us; pull 813 against 820), half storage 8.
 #ifndef LBM_STEP_MINB19
 #define LBM_STEP_MINB19 10
 #endif
@@ -1411,7 +1484,7 @@ static __global__ void __launch_bounds__(256) k_stats_total(const float* stats_w
 // STATS: also write the plane statistics of the state this step starts from (warp slot
 // blockIdx.x of each row, nxp/32 slots per row).
 template <int Q, class S, int CL, int LOAD, int STORE, bool STATS = false, int COLL = 0>
-__global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? 8 : LBM_STEP_MINB19) : LBM_STEP_MINB27)
+__global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? (acc_form<S> && STORE != 1 ? 9 : 8) : LBM_STEP_MINB19) : LBM_STEP_MINB27)
     k_step(const __grid_constant__ KParams p) {
   chain_begin();
   const int x = blockIdx.x * 32 + threadIdx.x;
