@@ -704,6 +704,31 @@ __device__ __forceinline__ V gelu_v(V a) {
 
 __device__ __forceinline__ float gelu_erf(float a) { return gelu_v<float>(a); }
 
+// The same by erf(z) = 1 - t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2), t = 1 / (1 + p z) for
+// z >= 0 (Abramowitz & Stegun, formula 7.1.26, after Hastings; absolute error below 1.5e-7), with
+// m = q t e - 1 = -(1 - erf|z|).  The closure step of half-storage lattices keeps it: another float32
+// rounding flips roundings of the stored values, and after some tens of steps the flow differs by
+// the storage rounding noise itself.
+template <class V>
+__device__ __forceinline__ V gelu_as(V a) {
+  using L = Lanes<V>;
+  V az, t, e;
+#pragma unroll
+  for (int k = 0; k < L::n; k++) L::put(az, k, fabsf(L::get(a, k)) * 0.70710678118654752f);  // |z|
+  const V den = vfma(az, vset<V>(0.3275911f), vset<V>(1.f));
+#pragma unroll
+  for (int k = 0; k < L::n; k++) L::put(t, k, __fdividef(1.f, L::get(den, k)));
+  V q = vfma(vset<V>(1.061405429f), t, vset<V>(-1.453152027f));
+  q = vfma(q, t, vset<V>(1.421413741f));
+  q = vfma(q, t, vset<V>(-0.284496736f));
+  q = vfma(q, t, vset<V>(0.254829592f));
+  const V arg = vmul(az, vmul(az, vset<V>(-1.4426950408889634f)));  // -z^2 log2(e)
+#pragma unroll
+  for (int k = 0; k < L::n; k++) L::put(e, k, ex2_approx(L::get(arg, k)));
+  const V m = vfma(vmul(q, t), e, vset<V>(-1.f));
+  return vfma(vmul(az, vset<V>(-0.70710678118654752f)), m, vmul(a, vset<V>(0.5f)));
+}
+
 // Orientation of the +/- pair (I, I+1), I odd: the member whose first non-zero velocity
 // component is positive is the primary one, so that c.u is a plain sum with a leading +.
 __host__ __device__ constexpr int lead(int i) { return cx(i) ? cx(i) : cy(i) ? cy(i) : cz(i); }

@@ -30,7 +30,7 @@
 // then undefined.
 //
 // Bound by instruction issue, most of it the 64 GELUs of a cell: with gelu_v in its logistic form
-// and bare reciprocals 512x256x256 D3Q19 FP32 takes 2188 -> 1792 us a step, 256x128x128 298 -> 250 us.
+// and bare reciprocals (FP32 storage) 512x256x256 D3Q19 takes 2188 -> 1792 us a step, 256x128x128 298 -> 250 us.
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -186,6 +186,10 @@ __global__ void __launch_bounds__(128 * MLP_NG, 1) k_step_mlp(const __grid_const
     __syncthreads();
     tc_fence_after();
   }
+  auto act = [](float2 a) {  // see gelu_as
+    if constexpr (acc_form<S>) return gelu_v(a);
+    else return gelu_as(a);
+  };
   const uint32_t tmem = sm.tmem;
   const uint32_t dcol = tmem + 32u * g;                          // this group's accumulator
   const uint32_t tl = dcol + ((uint32_t)((warp & 3) * 32) << 16);  // this warp's lanes
@@ -269,8 +273,8 @@ __global__ void __launch_bounds__(128 * MLP_NG, 1) k_step_mlp(const __grid_const
       tmem_ld16(tl + 16 * half, v);
 #pragma unroll
       for (int c = 0; c < 4; c++) {
-        const float2 g01 = gelu_v(make_float2(v[4 * c], v[4 * c + 1]));
-        const float2 g23 = gelu_v(make_float2(v[4 * c + 2], v[4 * c + 3]));
+        const float2 g01 = act(make_float2(v[4 * c], v[4 * c + 1]));
+        const float2 g23 = act(make_float2(v[4 * c + 2], v[4 * c + 3]));
         *reinterpret_cast<uint4*>(A + core_off<MLP_K2>(t, 16 * half + 4 * c)) =
             make_uint4(to_tf32(g01.x), to_tf32(g01.y), to_tf32(g23.x), to_tf32(g23.y));
       }
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(128 * MLP_NG, 1) k_step_mlp(const __grid_const
       tmem_ld16(tl + 16 * half, v);
 #pragma unroll
       for (int pr = 0; pr < 8; pr++)
-        acc = vfma(sm.W3[8 * half + pr], gelu_v(make_float2(v[2 * pr], v[2 * pr + 1])), acc);
+        acc = vfma(sm.W3[8 * half + pr], act(make_float2(v[2 * pr], v[2 * pr + 1])), acc);
     }
     const float yv = sm.b3 + (acc.x + acc.y);
     const float cs2 = fmaxf(softplus_f(yv) * p.cs2 * 1.4426950408889634f, p.cs2_min);  // / ln 2
