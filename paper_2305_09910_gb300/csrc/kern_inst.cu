@@ -64,8 +64,13 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       const long long extra = (p.nblist + per - 1) / per;
       const bool fused = p.nblist <= LBM_LIST_FUSE_MAX && g.z + extra <= 65535;
       if (fused) g.z += (unsigned)extra;
-      if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true>, g, L.block, L.stream, p);
-      else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true>, g, L.block, L.stream, p);
+      if (p.nx % 2 && p.face[1] == FACE_PERIODIC) {
+        if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true, true>, g, L.block, L.stream, p);
+        else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true, true>, g, L.block, L.stream, p);
+      } else {
+        if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true>, g, L.block, L.stream, p);
+        else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true>, g, L.block, L.stream, p);
+      }
       if (!fused) {
         const unsigned nb = (unsigned)((p.nblist + 127) / 128);
         if (closure == CL_NONE) launch_chained(k_step_list<Q, S, CL_NONE>, nb, 128, L.stream, p);

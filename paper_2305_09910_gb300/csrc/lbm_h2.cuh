@@ -57,13 +57,15 @@ __device__ __forceinline__ void outflow_fix2(const KParams& p, int x0, float (&f
   }
 }
 
-// Slot offsets of the two cells' sources in a direction with c_x != 0 (periodic x wrap).
+// Slot offsets of the two cells' sources in a direction with c_x != 0 (periodic x wrap).  LAST: the
+// row's last cell may be the first of its pair (odd nx, see k_step_h2), else it is always the second.
+template <bool LAST = false>
 __device__ __forceinline__ void xsrc(int c, const KParams& p, int x, int cell, int& ca, int& cb) {
   if (c > 0) {  // sources x-1, x
     ca = cell + (x == 0 ? p.nx : 0);
     cb = cell + 1;
   } else {       // sources x+1, x+2
-    ca = cell;
+    ca = cell - (LAST && x == p.nx - 1 ? p.nx : 0);
     cb = cell + 1 - (x + 1 == p.nx - 1 ? p.nx : 0);
   }
 }
@@ -199,7 +201,7 @@ __device__ __forceinline__ void own_outflow_masks(const KParams& p, int x, int c
 // the simple inflow/outflow face cells are updated here, the listed ones by k_step_list.  A lane with one interior cell loads both cells'
 // words (the other cell's sources, one x further, stay inside the arrays) and stores one half.
 // The packed loads of a lane whose two cells take the fast path.
-template <int Q, class S, int LOAD>
+template <int Q, class S, int LOAD, bool LAST = false>
 __device__ __forceinline__ void pair_loads(const KParams& p, int x, int cell, uint32_t (&h)[Q]) {
 #pragma unroll
   for (int i = 0; i < Q; i++) {
@@ -211,7 +213,7 @@ __device__ __forceinline__ void pair_loads(const KParams& p, int x, int cell, ui
         h[i] = chk(p, base + cell, 4, CHK_POP) ? ldh_u32(base + cell) : 0u;
       } else {
         int a, b;
-        xsrc(cx(i), p, x, cell, a, b);
+        xsrc<LAST>(cx(i), p, x, cell, a, b);
         const uint32_t lo = chk(p, base + a, 2, CHK_POP) ? ldh_u16(base + a) : 0u;
         const uint32_t hi = chk(p, base + b, 2, CHK_POP) ? ldh_u16(base + b) : 0u;
         h[i] = lo | (hi << 16);
@@ -258,7 +260,7 @@ __device__ __forceinline__ void xface_fix(const KParams& p, int x, int cell, boo
   }
 }
 
-template <int Q, class S, int CL, int LOAD, bool STATS, bool SPLIT>
+template <int Q, class S, int CL, int LOAD, bool STATS, bool SPLIT, bool LAST>
 __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z, int cell, int clsA, int clsB,
                                           bool fast, float (&v)[NSTAT], bool xfA, bool xfB) {
   constexpr bool PACKED = Q == 27 ? LBM_H2_PACKED27 : LBM_H2_PACKED19;
@@ -270,7 +272,7 @@ __device__ __forceinline__ void pair_pull(const KParams& p, int x, int y, int z,
     fast = true;
   }
   if (fast) {
-    pair_loads<Q, S, LOAD>(p, x, cell, h);
+    pair_loads<Q, S, LOAD, LAST>(p, x, cell, h);
   } else {
     uint32_t hs[Q];
     load_pair_rules<Q, S, LOAD>(p, x, y, z, cell, clsA | (xfA ? CLS_XFACE : 0), clsB | (xfB ? CLS_XFACE : 0), hs, &oa, &ob);
@@ -343,7 +345,10 @@ __device__ __noinline__ void list_cell(const KParams& p, long long t);
 #endif
 // STATS: also write the plane statistics of the state this step starts from (warp slot
 // blockIdx.x of each row, ceil(nxp/64) slots per row).
-template <int Q, class S, int CL, int LOAD, int STORE, bool STATS = false, bool SPLIT = false>
+// LAST (split step of odd rows with a periodic x seam): the row's last cell is an interior cell and
+// the first of its pair, and its sources with c_x = -1 wrap.  A form of its own, as the two selects cost
+// the even rows 1 % (1024x512x512 D3Q19 FP16, ten steps and moments 41.55 -> 41.97 ms).
+template <int Q, class S, int CL, int LOAD, int STORE, bool STATS = false, bool SPLIT = false, bool LAST = false>
 __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_step_h2(const __grid_constant__ KParams p) {
   static_assert(sizeof(S) == 2, "two 16-bit populations per word");
   chain_begin();
@@ -377,7 +382,7 @@ __global__ void __launch_bounds__(128, Q == 27 ? LBM_H2_MINB27 : LBM_H2_MINB) k_
 #pragma unroll
   for (int k = 0; k < NSTAT; k++) v[k] = 0.f;
   if constexpr (STORE == 2) {
-    pair_pull<Q, S, CL, LOAD, STATS, SPLIT>(p, x, y, z, cell, clsA, clsB, fast, v, xfA, xfB);
+    pair_pull<Q, S, CL, LOAD, STATS, SPLIT, LAST>(p, x, y, z, cell, clsA, clsB, fast, v, xfA, xfB);
   } else if constexpr (LOAD == 0) {
     pair_even<Q, S, CL, STATS>(p, x, cell, clsA, clsB, v);
   } else if (__all_sync(0xffffffffu, fast)) {
