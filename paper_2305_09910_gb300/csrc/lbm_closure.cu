@@ -672,31 +672,31 @@ lbm_status lbm_closure_samples(lbm_handle fine, double tau0_c, double cs0, const
   return LBM_OK;
 }
 
-// Scratch of a call that synchronises before it returns: one of SLOTS small device blocks that a
-// device keeps (2 KB, until the process ends), taken for the duration of the call by any thread
-// and stream, or stream-ordered memory where all are taken.  An allocation per call cost 0.1 ms:
-// the default pool gives its memory back at every synchronisation and maps 32 MB again.
+// Scratch of a call that synchronises before it returns: one of SLOTS small blocks in the module's
+// own device storage, taken for the duration of the call by any thread and stream, or stream-ordered
+// memory where all are taken.  An allocation per call cost 0.1 ms: the default pool gives its memory
+// back at every synchronisation and maps 32 MB again.  The storage lives and dies with the module in
+// its context, and its address is asked for by every call: after a device reset a kept one is stale.
+constexpr int SCRATCH_SLOTS = 64, SCRATCH_DOUBLES = 4;
+__device__ double call_scratch[SCRATCH_SLOTS * SCRATCH_DOUBLES];
+
 class CallScratch {
  public:
-  static constexpr int DOUBLES = 4;
   cudaError_t take(cudaStream_t st) {
+    void* mem = nullptr;
     cudaError_t e = cudaGetDevice(&dev_);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&mem, call_scratch);
     if (e != cudaSuccess) return e;
     if (dev_ < DEVICES) {
       std::lock_guard<std::mutex> hold(lock());
-      Kept& k = kept()[dev_];
-      if (!k.mem && cudaMalloc((void**)&k.mem, SLOTS * DOUBLES * sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        k.mem = nullptr;
-      }
-      for (int i = 0; k.mem && slot_ < 0 && i < SLOTS; i++)
-        if (!(k.used >> i & 1)) {
-          k.used |= 1ull << i;
+      for (int i = 0; slot_ < 0 && i < SCRATCH_SLOTS; i++)
+        if (!(used()[dev_] >> i & 1)) {
+          used()[dev_] |= 1ull << i;
           slot_ = i;
-          p = k.mem + i * DOUBLES;
+          p = static_cast<double*>(mem) + i * SCRATCH_DOUBLES;
         }
     }
-    return p ? cudaSuccess : cudaMallocAsync((void**)&p, DOUBLES * sizeof(double), st);
+    return p ? cudaSuccess : cudaMallocAsync((void**)&p, SCRATCH_DOUBLES * sizeof(double), st);
   }
   // after the call's work is queued; idle: the stream has been waited for
   void give(cudaStream_t st, bool idle) {
@@ -704,25 +704,21 @@ class CallScratch {
       if (p) cudaFreeAsync(p, st);
     } else if (idle) {  // after an error the slot stays taken: its work may still be running
       std::lock_guard<std::mutex> hold(lock());
-      kept()[dev_].used &= ~(1ull << slot_);
+      used()[dev_] &= ~(1ull << slot_);
     }
     p = nullptr;
   }
   double* p = nullptr;
 
  private:
-  static constexpr int DEVICES = 64, SLOTS = 64;
-  struct Kept {
-    double* mem = nullptr;
-    uint64_t used = 0;
-  };
+  static constexpr int DEVICES = 64;
   static std::mutex& lock() {
     static std::mutex m;
     return m;
   }
-  static Kept* kept() {
-    static Kept k[DEVICES];
-    return k;
+  static uint64_t* used() {  // a bit per slot and device
+    static uint64_t u[DEVICES];
+    return u;
   }
   int dev_ = 0, slot_ = -1;
 };
@@ -798,7 +794,7 @@ lbm_status lbm_closure_loss_grad(const float* params, const float* x, const floa
   cudaError_t e = backward_grid(n, &grid);
   if (e == cudaSuccess) e = scratch.take(st);
   double* const sums = scratch.p;
-  if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, CallScratch::DOUBLES * sizeof(double), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, SCRATCH_DOUBLES * sizeof(double), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, MLP_NPARAM * sizeof(float), st);
   if (e == cudaSuccess && n > 0) {
     BackArgs a{};
