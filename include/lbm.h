@@ -263,8 +263,10 @@ lbm_status lbm_step(lbm_handle h, int64_t n);
  * the step then waited again, with a longer bound, for the tensor core to finish and completed
  * its tiles); or that second wait gave up as well, after which the tensor-core work may still
  * have been running when the results were read and the kernel left: the handle is then marked
- * unusable and every later step returns LBM_ECUDA (likewise when a multi-step launch gave up a
- * bounded wait for its own blocks); or, in a library built with
+ * unusable, every later step returns LBM_ECUDA, and so do lbm_reduce, lbm_stats_get and the exports
+ * to host arrays, after they have written their results (likewise when a multi-step launch gave
+ * up a bounded wait for its own blocks and ended between two steps, which all of these calls notice
+ * by themselves); or, in a library built with
  * LBM_BOUNDS_CHECK (liblbm_check.so), a kernel skipped an access outside its array. */
 lbm_status lbm_sync(lbm_handle h);
 
@@ -273,7 +275,8 @@ lbm_status lbm_sync(lbm_handle h);
  * default 2^22 (far longer than any MMA takes), polls = -1 restores it, 0 makes every first
  * wait give up at once, which drives the timeout path of lbm_sync without a device fault
  * (the step still waits, with the full bound, for the tensor core to finish before it reads
- * the results).  EINVAL outside [-1, 2^22].  Failure detection; the paper has no
+ * the results).  The same limit holds for the waits of a multi-step launch for its own blocks
+ * (lbm_step on small lattices): with 0 it ends after its first step.  EINVAL outside [-1, 2^22].  Failure detection; the paper has no
  * counterpart. */
 lbm_status lbm_debug_set_wait_polls(lbm_handle h, int64_t polls);
 

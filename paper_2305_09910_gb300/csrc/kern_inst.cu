@@ -118,7 +118,7 @@ cudaError_t launch_step(const KParams& p, int closure, int mode, const Launch& L
 // the row segments over the SMs once, up to 16; the grid is at most what fits on the device at
 // once (a cooperative launch refuses more, it never waits).
 template <int Q, class S, int CL, int COLL, bool AA>
-static cudaError_t multi_one(const KParams2& pp, int nsteps, int odd0, unsigned* count, cudaStream_t stream, int nsm) {
+static cudaError_t multi_one(const KParams2& pp, int nsteps, int odd0, unsigned* count, int* alarm, cudaStream_t stream, int nsm) {
   auto kern = k_step_multi<Q, S, CL, COLL, AA>;
   const KParams& p = pp.p[0];
   const long long nseg = (long long)(p.nxp / 32) * p.ny * p.nz;
@@ -130,35 +130,35 @@ static cudaError_t multi_one(const KParams2& pp, int nsteps, int odd0, unsigned*
   const int blocks = (int)std::min<long long>((nseg + warps - 1) / warps, (long long)per_sm * nsm);
   e = cudaMemsetAsync(count, 0, sizeof(unsigned), stream);
   if (e != cudaSuccess) return e;
-  void* args[] = {(void*)&pp, (void*)&nsteps, (void*)&odd0, (void*)&count};
+  void* args[] = {(void*)&pp, (void*)&nsteps, (void*)&odd0, (void*)&count, (void*)&alarm};
   return cudaLaunchCooperativeKernel((const void*)kern, dim3(blocks), dim3(32, warps), args, 0, stream);
 }
 
 template <int Q, class S, int COLL, bool AA>
-static cudaError_t multi_cl(const KParams2& pp, int closure, int nsteps, int odd0, unsigned* count, cudaStream_t st,
+static cudaError_t multi_cl(const KParams2& pp, int closure, int nsteps, int odd0, unsigned* count, int* alarm, cudaStream_t st,
                             int nsm) {
-  return closure == CL_NONE ? multi_one<Q, S, CL_NONE, COLL, AA>(pp, nsteps, odd0, count, st, nsm)
-                            : multi_one<Q, S, CL_SMAG, COLL, AA>(pp, nsteps, odd0, count, st, nsm);
+  return closure == CL_NONE ? multi_one<Q, S, CL_NONE, COLL, AA>(pp, nsteps, odd0, count, alarm, st, nsm)
+                            : multi_one<Q, S, CL_SMAG, COLL, AA>(pp, nsteps, odd0, count, alarm, st, nsm);
 }
 
 template <int Q, class S, bool AA>
 static cudaError_t multi_coll(const KParams2& pp, int closure, int coll, int nsteps, int odd0, unsigned* count,
-                              cudaStream_t st, int nsm) {
+                              int* alarm, cudaStream_t st, int nsm) {
   if constexpr (Q == 19) {
-    if (coll == 1) return multi_cl<Q, S, 1, AA>(pp, closure, nsteps, odd0, count, st, nsm);
+    if (coll == 1) return multi_cl<Q, S, 1, AA>(pp, closure, nsteps, odd0, count, alarm, st, nsm);
   }
-  if (coll == 2) return multi_cl<Q, S, 2, AA>(pp, closure, nsteps, odd0, count, st, nsm);
-  return multi_cl<Q, S, 0, AA>(pp, closure, nsteps, odd0, count, st, nsm);
+  if (coll == 2) return multi_cl<Q, S, 2, AA>(pp, closure, nsteps, odd0, count, alarm, st, nsm);
+  return multi_cl<Q, S, 0, AA>(pp, closure, nsteps, odd0, count, alarm, st, nsm);
 }
 
 template <int Q, class S>
 cudaError_t launch_step_multi(const KParams& p0, const KParams& p1, int closure, int coll, bool aa, int odd0,
-                              int nsteps, unsigned* count, cudaStream_t stream, int nsm) {
+                              int nsteps, unsigned* count, int* alarm, cudaStream_t stream, int nsm) {
   KParams2 pp;
   pp.p[0] = p0;
   pp.p[1] = p1;
-  return aa ? multi_coll<Q, S, true>(pp, closure, coll, nsteps, odd0, count, stream, nsm)
-            : multi_coll<Q, S, false>(pp, closure, coll, nsteps, odd0, count, stream, nsm);
+  return aa ? multi_coll<Q, S, true>(pp, closure, coll, nsteps, odd0, count, alarm, stream, nsm)
+            : multi_coll<Q, S, false>(pp, closure, coll, nsteps, odd0, count, alarm, stream, nsm);
 }
 
 template <int Q, class S, int LOAD, int STORE>
@@ -258,6 +258,6 @@ template cudaError_t launch_export<LBM_Q, LBM_S>(const KParams&, int, int, const
 template cudaError_t launch_init_eq<LBM_Q, LBM_S>(const KParams&, const float*, const float*, const Launch&);
 template cudaError_t launch_set_pop<LBM_Q, LBM_S>(const KParams&, const float*, const Launch&);
 template cudaError_t launch_step_multi<LBM_Q, LBM_S>(const KParams&, const KParams&, int, int, bool, int, int,
-                                                     unsigned*, cudaStream_t, int);
+                                                     unsigned*, int*, cudaStream_t, int);
 
 }  // namespace lbm

@@ -33,7 +33,7 @@ struct lbm_s {
   int* status = nullptr;      // device status word
   unsigned* arrivals = nullptr; // barrier arrivals of k_step_multi
   int* chk_bad = nullptr;     // first out-of-range access seen by a bounds-checked build
-  int* status_host = nullptr; // pinned copy
+  int* status_host = nullptr; // pinned: the copy, and behind it the alarm word of k_step_multi
   double* sums = nullptr;     // 4 doubles (lbm_reduce)
   double* partial = nullptr;  // nz * ny * 10 doubles: per-row sums of the reductions
   float* stats_w = nullptr;   // per-warp plane statistics of sampling steps (see ensure_stats_w)
@@ -61,8 +61,8 @@ struct lbm_s {
   int nat_valid = 1;          // natural layout came from an import (outflow slots hold values)
   int prev_post = 0;          // pull: the other array holds the post-collision state before the current one
   int nsm = 0;                // multiprocessors of the device (persistent grid size)
-  int wait_polls = MBAR_POLLS; // polls of the closure step's first wait for each tile's MMA
-  bool broken = false;        // a device wait gave up twice: results and device state undefined
+  int wait_polls = MBAR_POLLS; // polls of the closure step's first wait for each tile's MMA and of k_step_multi's barriers
+  bool broken = false;        // a device wait gave up for good: results and device state undefined
   std::string err;
 };
 
@@ -378,9 +378,9 @@ static cudaError_t dispatch_multi(const lbm_s* h, const KParams& p0, const KPara
   const int odd0 = aa ? h->parity : 0;
   const int cl = h->prm.closure, coll = h->prm.collision;
   switch (h->prm.precision) {
-    case LBM_F32: return launch_step_multi<Q, float>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
-    case LBM_F16_SHIFTED: return launch_step_multi<Q, __half>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
-    default: return launch_step_multi<Q, __nv_bfloat16>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->stream, h->nsm);
+    case LBM_F32: return launch_step_multi<Q, float>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->status_host + 1, h->stream, h->nsm);
+    case LBM_F16_SHIFTED: return launch_step_multi<Q, __half>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->status_host + 1, h->stream, h->nsm);
+    default: return launch_step_multi<Q, __nv_bfloat16>(p0, p1, cl, coll, aa, odd0, nsteps, h->arrivals, h->status_host + 1, h->stream, h->nsm);
   }
 }
 
@@ -651,7 +651,8 @@ lbm_status lbm_create(int nx, int ny, int nz, int stencil, double tau, const lbm
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->sums, 4 * sizeof(double), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->partial, (size_t)ny * nz * 10 * sizeof(double), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->stats, (size_t)ny * LBM_STATS_K * sizeof(double), h->stream);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->status_host, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->status_host, 2 * sizeof(int));
+  if (e == cudaSuccess) h->status_host[1] = 0;
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f, 0, fbytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, (size_t)gplane, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), h->stream);
@@ -799,6 +800,17 @@ static lbm_status ensure_stats_w(lbm_handle h) {
   const size_t slots = (size_t)((h->nxp + 31) / 32) * h->ny * h->nz;
   CUDA_TRY(h, cudaMallocAsync((void**)&h->stats_w, slots * 10 * sizeof(float), h->stream));
   return LBM_OK;
+}
+
+static const char* const BROKEN_MSG =
+    "the handle is unusable: a learned-closure step gave up waiting for the tensor core twice, or a "
+    "multi-step launch for its blocks";
+
+// LBM_ECUDA on a handle whose state a wait that gave up has left between two steps; of a
+// multi-step launch every call knows that has waited for the stream (the launch writes it to host memory).
+static lbm_status check_broken(lbm_handle h) {
+  if (static_cast<volatile int*>(h->status_host)[1]) h->broken = true;
+  return h->broken ? fail(h, LBM_ECUDA, "%s", BROKEN_MSG) : LBM_OK;
 }
 
 // n steps; with every > 0 the plane statistics of the state each step k (k % every == 0)
@@ -964,13 +976,9 @@ static int64_t run_multi(lbm_handle h, int64_t n) {
   return n;
 }
 
-static const char* const BROKEN_MSG =
-    "the handle is unusable: a learned-closure step gave up waiting for the tensor core twice, or a "
-    "multi-step launch for its blocks";
-
 lbm_status lbm_step(lbm_handle h, int64_t n) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
-  if (h->broken) return fail(h, LBM_ECUDA, "%s", BROKEN_MSG);
+  if (check_broken(h) != LBM_OK) return LBM_ECUDA;
   if (n < 0) return fail(h, LBM_EINVAL, "n must be >= 0");
   if (h->prm.closure == LBM_CLOSURE_MLP && !h->mlp_set)
     return fail(h, LBM_ESTATE, "MLP closure selected but lbm_set_closure was not called");
@@ -1000,7 +1008,7 @@ lbm_status lbm_step(lbm_handle h, int64_t n) {
 
 lbm_status lbm_step_stats(lbm_handle h, int64_t n, int64_t every) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
-  if (h->broken) return fail(h, LBM_ECUDA, "%s", BROKEN_MSG);
+  if (check_broken(h) != LBM_OK) return LBM_ECUDA;
   if (n < 0) return fail(h, LBM_EINVAL, "n must be >= 0");
   if (every < 1) return fail(h, LBM_EINVAL, "every must be >= 1");
   return run_steps(h, n, every);
@@ -1200,10 +1208,9 @@ lbm_status lbm_sync(lbm_handle h) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
   CUDA_TRY(h, cudaMemcpyAsync(h->status_host, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  if (*h->status_host & (4 | MULTI_GAVE_UP)) {
-    h->broken = true;
-    return fail(h, LBM_ECUDA, "%s", BROKEN_MSG);
-  }
+  if (*h->status_host & 4) h->broken = true;
+  const lbm_status s = check_broken(h);
+  if (s != LBM_OK) return s;
   if (*h->status_host & 2)
     return fail(h, LBM_ECUDA,
                 "a learned-closure step gave up waiting for its tensor-core result (then waited with the full bound)");
@@ -1262,6 +1269,7 @@ lbm_status lbm_moments(lbm_handle h, float* rho, float* u, int on_device) {
     if (trho) cudaFreeAsync(trho, h->stream);
     if (tu) cudaFreeAsync(tu, h->stream);
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return check_broken(h);
   }
   return LBM_OK;
 }
@@ -1300,6 +1308,7 @@ static lbm_status get_pop(lbm_handle h, float* df, int on_device, bool raw) {
       cudaFreeAsync(t, h->stream);
     }
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return check_broken(h);
   }
   return LBM_OK;
 }
@@ -1314,7 +1323,7 @@ lbm_status lbm_reduce(lbm_handle h, double out[4]) {
   if (s != LBM_OK) return s;
   CUDA_TRY(h, cudaMemcpyAsync(out, h->sums, 4 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return LBM_OK;
+  return check_broken(h);
 }
 
 lbm_status lbm_stats_reset(lbm_handle h) {
@@ -1342,7 +1351,7 @@ lbm_status lbm_stats_get(lbm_handle h, double* out, int64_t* nsamples) {
                               cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   if (nsamples) *nsamples = h->nsamples;
-  return LBM_OK;
+  return check_broken(h);
 }
 
 lbm_status lbm_set_closure(lbm_handle h, const uint16_t* bf16_params, int n, double scale_pi,

@@ -108,7 +108,8 @@ struct KParams {
   int split;             // the pull gather step runs as the interior x-pair step + k_step_list
   int* status;           // bit 0: non-finite or non-positive density seen; bits 1, 2: a
                          // bounded wait of the learned-closure step gave up (once, twice)
-  int wait_polls;        // polls of the closure step's first wait for each tile's MMA
+  int wait_polls;        // polls of the closure step's first wait for each tile's MMA, and of
+                         // a grid barrier's wait in k_step_multi (each a read of the L2)
   float* stats_w;        // sampling steps: per-warp plane sums, [(z ny + y) nws + ws][10]
   long long plane;       // nxp * ny * nz
   int nx, ny, nz, nxp;
@@ -1549,7 +1550,8 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? (acc_form<S> && ST
 // one in registers, so that a step goes straight to its gather.  Blocks are as large as spreads
 // the segments evenly over the SMs (few arrivals per barrier).  Two-grid pull alternates the two
 // arrays (pp.p[s & 1]); AA alternates the even and odd forms on one array, starting with the form
-// `odd0`.  Every cell gets the bits of the single-launch step.
+// `odd0`.  Every cell gets the bits of the single-launch step.  A block whose bounded wait gives up
+// sets *alarm and leaves, and the others after it.
 // Bound by latency: a step of a lattice of one segment per warp is one gather from the L2, the
 // collision's dependent chain, the store and the barrier (3.5 us at 32x16x16 cells).  64x32x32
 // D3Q19 FP32: AA 5.9 -> 4.5, pull 4.75 -> 4.2 us a step (before: blocks of 4 warps, the class read
@@ -1558,8 +1560,6 @@ struct KParams2 {
   KParams p[2];
 };
 constexpr int MULTI_WARPS = 16;          // warps of a block at most
-constexpr int MULTI_GAVE_UP = 8;         // status bit 3: a barrier wait gave up, the launch ended early
-constexpr int MULTI_POLLS = 1 << 22;     // polls of a barrier wait (each a read of the L2)
 
 template <int Q, class S, int CL, int LOAD, int STORE, int COLL>
 __device__ __forceinline__ void step_segment(const KParams& p, int x, int y, int z, int cbyte) {
@@ -1580,17 +1580,18 @@ __device__ __forceinline__ void step_segment(const KParams& p, int x, int y, int
 }
 
 // Arrival and wait of one block at a grid-wide barrier (count: arrivals so far, zeroed before the
-// launch); false when the bounded wait gave up.
-__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, bool* dead) {
+// launch); false when the bounded wait gave up (at once with a limit of 0 polls).
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int polls, bool* dead) {
   __syncthreads();
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
-    unsigned v = 0;
-    int it = 0;
-    do {
+    bool here = false;
+    for (int it = 0; !here && it < polls; it++) {
+      unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-    } while ((int)(v - target) < 0 && ++it < MULTI_POLLS);
-    *dead = (int)(v - target) < 0;
+      here = (int)(v - target) >= 0;
+    }
+    *dead = !here;
   }
   __syncthreads();
   return !*dead;
@@ -1598,7 +1599,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, b
 
 template <int Q, class S, int CL, int COLL, bool AA>
 __global__ void __launch_bounds__(32 * MULTI_WARPS, Q == 19 ? 2 : 1)
-    k_step_multi(const __grid_constant__ KParams2 pp, int nsteps, int odd0, unsigned* count) {
+    k_step_multi(const __grid_constant__ KParams2 pp, int nsteps, int odd0, unsigned* count, volatile int* alarm) {
   __shared__ bool dead;
   const KParams& p0 = pp.p[0];
   const int wpr = p0.nxp / 32, nseg = wpr * p0.ny * p0.nz;
@@ -1629,8 +1630,8 @@ __global__ void __launch_bounds__(32 * MULTI_WARPS, Q == 19 ? 2 : 1)
         step_segment<Q, S, CL, 2, 2, COLL>(p0, x, y, z, c);
       }
     }
-    if (s + 1 < nsteps && !grid_barrier(count, (unsigned)(s + 1) * gridDim.x, &dead)) {
-      if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(p0.status, MULTI_GAVE_UP);
+    if (s + 1 < nsteps && !grid_barrier(count, (unsigned)(s + 1) * gridDim.x, p0.wait_polls, &dead)) {
+      if (threadIdx.x == 0 && threadIdx.y == 0) *alarm = 1;  // host memory: every call that waits reads it
       return;
     }
   }

@@ -41,7 +41,7 @@ template <int Q, class S>
 cudaError_t launch_set_pop(const KParams& p, const float* df, const Launch& L);
 template <int Q, class S>
 cudaError_t launch_step_multi(const KParams& p0, const KParams& p1, int closure, int coll, bool aa, int odd0,
-                              int nsteps, unsigned* count, cudaStream_t stream, int nsm);
+                              int nsteps, unsigned* count, int* alarm, cudaStream_t stream, int nsm);
 
 #define LBM_DECLARE_INSTANCE(Q, S)                                                                 \
   extern template cudaError_t launch_step<Q, S>(const KParams&, int, int, const Launch&, bool, int*, int); \
@@ -52,7 +52,7 @@ cudaError_t launch_step_multi(const KParams& p0, const KParams& p1, int closure,
                                                    const Launch&);                                 \
   extern template cudaError_t launch_set_pop<Q, S>(const KParams&, const float*, const Launch&);     \
   extern template cudaError_t launch_step_multi<Q, S>(const KParams&, const KParams&, int, int, bool, int, \
-                                                      int, unsigned*, cudaStream_t, int);
+                                                      int, unsigned*, int*, cudaStream_t, int);
 
 LBM_DECLARE_INSTANCE(19, float)
 LBM_DECLARE_INSTANCE(19, __half)
