@@ -32,20 +32,35 @@ static bool odd_pairs(const KParams& p) {
   return (p.nxp + 63) / 64 >= 11 * (p.nx & 1) + 23 * faces;
 }
 
+// Step launches are chained (programmatic stream serialisation), in graph replays only where the grid
+// takes about a wave of blocks or more, 8 per SM of the one-cell kernel, 6 of the pairs (D3Q27: 3).  Below, the
+// blocks of a chained step find free places on every SM beside those of the step before, and its last
+// ones go where these end first, so that SMs end up with uneven shares; launched one by one such steps
+// wait for the host anyhow (2:1 refined box 64x32x32 FP16 with nine launches 31.7 us chained, 33-35
+// not).  Replays, us a step, chained / not: D3Q19 FP32 AA box 64x50x46 (1196 blocks) 5.4 / 4.9, channel
+// 32x80x90 (1800) 9.8 / 9.9; D3Q27 FP32 32x50x60 (780) AA box 6.1 / 5.0, pull channel 13.0 / 10.8; FP16
+// pull pairs 64x50x46 (598) 6.2 / 5.9, 128x48x48 (1152) 8.5 / 8.7, D3Q27 64x40x38 (380) 7.9 / 7.7,
+// 100x40x30 (600) 8.5 / 9.0.
+static void launch_step_grid(void (*kern)(KParams), dim3 g, const Launch& L, int wave, const KParams& p) {
+  const bool chain = !L.replay || (long long)g.x * g.y * g.z > (long long)wave * L.nsm;
+  launch_chained(chain, kern, g, L.block, L.stream, p);
+}
+constexpr int WAVE_CELLS = 8, WAVE_PAIRS = LBM_Q == 27 ? 3 : 6;
+
 template <int Q, class S, int LOAD, int STORE, bool STATS>
 static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll, int* nws) {
   if constexpr (Q == 19) {
     if (coll == 1) {
       if (nws) *nws = p.nxp / 32;
-      if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 1>, L.grid, L.block, L.stream, p);
-      else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 1>, L.grid, L.block, L.stream, p);
+      if (closure == CL_NONE) launch_step_grid(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 1>, L.grid, L, WAVE_CELLS, p);
+      else launch_step_grid(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 1>, L.grid, L, WAVE_CELLS, p);
       return;
     }
   }
   if (coll == 2) {  // regularised collision: one cell per thread, every stencil and storage
     if (nws) *nws = p.nxp / 32;
-    if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 2>, L.grid, L.block, L.stream, p);
-    else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 2>, L.grid, L.block, L.stream, p);
+    if (closure == CL_NONE) launch_step_grid(k_step<Q, S, CL_NONE, LOAD, STORE, STATS, 2>, L.grid, L, WAVE_CELLS, p);
+    else launch_step_grid(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS, 2>, L.grid, L, WAVE_CELLS, p);
     return;
   }
   // half storage, gather step of two-grid pull without statistics (both stencils; D3Q19 unless
@@ -65,16 +80,16 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       const bool fused = p.nblist <= LBM_LIST_FUSE_MAX && g.z + extra <= 65535;
       if (fused) g.z += (unsigned)extra;
       if (p.nx % 2 && p.face[1] == FACE_PERIODIC) {
-        if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true, true>, g, L.block, L.stream, p);
-        else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true, true>, g, L.block, L.stream, p);
+        if (closure == CL_NONE) launch_step_grid(k_step_h2<Q, S, CL_NONE, 2, 2, false, true, true>, g, L, WAVE_PAIRS, p);
+        else launch_step_grid(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true, true>, g, L, WAVE_PAIRS, p);
       } else {
-        if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, 2, 2, false, true>, g, L.block, L.stream, p);
-        else launch_chained(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true>, g, L.block, L.stream, p);
+        if (closure == CL_NONE) launch_step_grid(k_step_h2<Q, S, CL_NONE, 2, 2, false, true>, g, L, WAVE_PAIRS, p);
+        else launch_step_grid(k_step_h2<Q, S, CL_SMAG, 2, 2, false, true>, g, L, WAVE_PAIRS, p);
       }
       if (!fused) {
         const unsigned nb = (unsigned)((p.nblist + 127) / 128);
-        if (closure == CL_NONE) launch_chained(k_step_list<Q, S, CL_NONE>, nb, 128, L.stream, p);
-        else launch_chained(k_step_list<Q, S, CL_SMAG>, nb, 128, L.stream, p);
+        if (closure == CL_NONE) launch_chained(true, k_step_list<Q, S, CL_NONE>, nb, 128, L.stream, p);
+        else launch_chained(true, k_step_list<Q, S, CL_SMAG>, nb, 128, L.stream, p);
       }
       return;
     }
@@ -85,14 +100,14 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       dim3 g = L.grid;
       g.x = (p.nxp + 63) / 64;
       if (nws) *nws = (int)g.x;
-      if (closure == CL_NONE) launch_chained(k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS>, g, L.block, L.stream, p);
-      else launch_chained(k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS>, g, L.block, L.stream, p);
+      if (closure == CL_NONE) launch_step_grid(k_step_h2<Q, S, CL_NONE, LOAD, STORE, STATS>, g, L, WAVE_PAIRS, p);
+      else launch_step_grid(k_step_h2<Q, S, CL_SMAG, LOAD, STORE, STATS>, g, L, WAVE_PAIRS, p);
       return;
     }
   }
   if (nws) *nws = p.nxp / 32;
-  if (closure == CL_NONE) launch_chained(k_step<Q, S, CL_NONE, LOAD, STORE, STATS>, L.grid, L.block, L.stream, p);
-  else launch_chained(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS>, L.grid, L.block, L.stream, p);
+  if (closure == CL_NONE) launch_step_grid(k_step<Q, S, CL_NONE, LOAD, STORE, STATS>, L.grid, L, WAVE_CELLS, p);
+  else launch_step_grid(k_step<Q, S, CL_SMAG, LOAD, STORE, STATS>, L.grid, L, WAVE_CELLS, p);
 }
 
 template <int Q, class S, int LOAD, int STORE>

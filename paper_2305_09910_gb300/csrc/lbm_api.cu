@@ -103,6 +103,8 @@ static Launch launch_cfg(const lbm_s* h) {
   L.block = dim3(32, 4, 1);
   L.grid = dim3(h->nxp / 32, (h->ny + 3) / 4, h->nz);
   L.stream = h->stream;
+  L.nsm = h->nsm;
+  L.replay = h->cap && h->stream == h->cap;
   return L;
 }
 
@@ -1169,9 +1171,9 @@ lbm_status lbm_refine_explode(lbm_handle coarse, int coarse_face, lbm_handle fin
   const long long n = (long long)nd * fine->nx * fine->ny;
   const int blocks = (int)std::min<long long>((n + 255) / 256, (long long)fine->nsm * 8);
   if (fine->prm.precision == LBM_F32)
-    launch_chained(k_refine_explode<uint32_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
+    launch_chained(true, k_refine_explode<uint32_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
   else
-    launch_chained(k_refine_explode<uint16_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
+    launch_chained(true, k_refine_explode<uint16_t>, blocks, 256, fine->stream, rp, nd, fine->nx, fine->ny, fine->nxp, coarse->nxp, substep);
   CUDA_TRY(fine, cudaGetLastError());
   return stream_join(fine, coarse, fine);
 }
@@ -1191,13 +1193,13 @@ lbm_status lbm_refine_coalesce(lbm_handle fine, int fine_face, lbm_handle coarse
   const int blocks = (int)std::min<long long>((n + 255) / 256, (long long)coarse->nsm * 8);
   switch (coarse->prm.precision) {
     case LBM_F32:
-      launch_chained(k_refine_coalesce<float>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
+      launch_chained(true, k_refine_coalesce<float>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
     case LBM_F16_SHIFTED:
-      launch_chained(k_refine_coalesce<__half>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
+      launch_chained(true, k_refine_coalesce<__half>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
     default:
-      launch_chained(k_refine_coalesce<__nv_bfloat16>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
+      launch_chained(true, k_refine_coalesce<__nv_bfloat16>, blocks, 256, coarse->stream, rp, nd, coarse->nx, coarse->ny, coarse->nxp, fine->nxp);
       break;
   }
   CUDA_TRY(coarse, cudaGetLastError());

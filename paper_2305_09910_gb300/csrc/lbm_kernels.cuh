@@ -1374,8 +1374,8 @@ __device__ __forceinline__ V collide(const KParams& p, V (&f)[Q], Macro<V>* mout
 }
 
 // ---- chained launches -----------------------------------------------------------------------
-// Step and transfer kernels are launched with programmatic stream serialisation: the blocks of a
-// launch may take the places that the last blocks of the one before leave free, and wait here until
+// Step kernels (not all of them, see launch_step_grid) and transfer kernels are launched with
+// programmatic stream serialisation: the blocks of a launch may take the places that the last blocks of the one before leave free, and wait here until
 // that one has finished and its writes are visible.  Nothing is read before.
 // 2:1 refined box 256x128x128 (nine launches per coarse step, six of them transfers of a few us),
 // three coarse steps and the exports: 2973 -> 2910 us; 64^3 AA steps replayed as a graph 10.4 -> 10.1 us.

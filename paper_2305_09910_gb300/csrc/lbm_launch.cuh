@@ -11,11 +11,13 @@ namespace lbm {
 struct Launch {
   dim3 grid, block;
   cudaStream_t stream;
+  int nsm;
+  bool replay;  // captured for lbm_step's graph
 };
 
-// Launch of a kernel that begins with chain_begin().
+// Launch of a kernel that begins with chain_begin(), chained to the launch before if `chain`.
 template <class... P, class... A>
-inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t stream, A&&... args) {
+inline void launch_chained(bool chain, void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t stream, A&&... args) {
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -24,7 +26,7 @@ inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, cudaStream
   cfg.blockDim = block;
   cfg.stream = stream;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = chain ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // (the callers read cudaGetLastError)
 }
 
