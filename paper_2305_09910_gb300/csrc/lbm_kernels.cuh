@@ -1548,7 +1548,7 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? (acc_form<S> && ST
 // launch, the steps separated by grid-wide barriers.  A warp owns the 32-cell row segments wid,
 // wid + W, ... of the lattice for the whole launch, and keeps the place and class of its first
 // one in registers, so that a step goes straight to its gather.  Blocks are as large as spreads
-// the segments evenly over the SMs (few arrivals per barrier).  Two-grid pull alternates the two
+// the segments evenly over the SMs (few arrivals per barrier; see multi_one).  Two-grid pull alternates the two
 // arrays (pp.p[s & 1]); AA alternates the even and odd forms on one array, starting with the form
 // `odd0`.  Every cell gets the bits of the single-launch step.  A block whose bounded wait gives up
 // sets *alarm and leaves, and the others after it.
@@ -1559,7 +1559,13 @@ __global__ void __launch_bounds__(128, Q == 19 ? (COLL == 1 ? (acc_form<S> && ST
 struct KParams2 {
   KParams p[2];
 };
-constexpr int MULTI_WARPS = 16;          // warps of a block at most
+// Warps of a block at most; two such blocks are resident per SM (multi_cap).  D3Q27 at 85 registers:
+// with 16 warps per SM at 128 a lattice of 2,433 to 3,648 segments took a second pass (64x40x38 FP32
+// pull channel 8.6 -> 6.0 us a step, AA 9.1 -> 6.7).
+template <int Q>
+constexpr int MULTI_WARPS = Q == 19 ? 16 : 12;
+template <int Q>
+constexpr int multi_cap(int nsm) { return 2 * MULTI_WARPS<Q> * nsm; }  // warps resident at once
 
 template <int Q, class S, int CL, int LOAD, int STORE, int COLL>
 __device__ __forceinline__ void step_segment(const KParams& p, int x, int y, int z, int cbyte) {
@@ -1598,7 +1604,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, i
 }
 
 template <int Q, class S, int CL, int COLL, bool AA>
-__global__ void __launch_bounds__(32 * MULTI_WARPS, Q == 19 ? 2 : 1)
+__global__ void __launch_bounds__(32 * MULTI_WARPS<Q>, 2)
     k_step_multi(const __grid_constant__ KParams2 pp, int nsteps, int odd0, unsigned* count, volatile int* alarm) {
   __shared__ bool dead;
   const KParams& p0 = pp.p[0];
