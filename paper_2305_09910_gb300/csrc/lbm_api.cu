@@ -33,7 +33,9 @@ struct lbm_s {
   int* status = nullptr;      // device status word
   unsigned* arrivals = nullptr; // barrier arrivals of k_step_multi
   int* chk_bad = nullptr;     // first out-of-range access seen by a bounds-checked build
-  int* status_host = nullptr; // pinned: the copy, and behind it the alarm word of k_step_multi
+  int* status_host = nullptr; // pinned: the copy, behind it the alarm word of k_step_multi and
+  int* seen_host = nullptr;   // what lbm_set_flags saw (two words)
+  bool solids = false;        // some cell is not fluid
   double* sums = nullptr;     // 4 doubles (lbm_reduce)
   double* partial = nullptr;  // nz * ny * 10 doubles: per-row sums of the reductions
   float* stats_w = nullptr;   // per-warp plane statistics of sampling steps (see ensure_stats_w)
@@ -248,15 +250,17 @@ static cudaError_t dispatch_set_pop(const lbm_s* h, const KParams& p, const floa
 
 // ---- small kernels of the set-up path -----------------------------------------------------
 
-// Copies dense flags into the padded layout and counts values outside the cell enum.
-__global__ void k_flags_in(const uint8_t* in, uint8_t* out, int nx, int ny, int nz, int nxp, int* bad) {
+// Copies dense flags into the padded layout; seen[0] += values outside the cell enum, seen[1] = 1 if a
+// cell is not fluid.
+__global__ void k_flags_in(const uint8_t* in, uint8_t* out, int nx, int ny, int nz, int nxp, int* seen) {
   const long long n = (long long)nx * ny * nz;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
        k += (long long)gridDim.x * blockDim.x) {
     const int x = (int)(k % nx);
     const long long r = k / nx;
     const uint8_t v = in[k];
-    if (v > CELL_INFLOW) atomicAdd(bad, 1);
+    if (v > CELL_INFLOW) atomicAdd(seen, 1);
+    if (v != CELL_FLUID) seen[1] = 1;
     out[r * nxp + x] = v > CELL_INFLOW ? (uint8_t)CELL_SOLID : v;
   }
 }
@@ -653,8 +657,11 @@ lbm_status lbm_create(int nx, int ny, int nz, int stencil, double tau, const lbm
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->sums, 4 * sizeof(double), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->partial, (size_t)ny * nz * 10 * sizeof(double), h->stream);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&h->stats, (size_t)ny * LBM_STATS_K * sizeof(double), h->stream);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->status_host, 2 * sizeof(int));
-  if (e == cudaSuccess) h->status_host[1] = 0;
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->status_host, 4 * sizeof(int));
+  if (e == cudaSuccess) {
+    h->status_host[1] = 0;
+    h->seen_host = h->status_host + 2;
+  }
   if (e == cudaSuccess) e = cudaMemsetAsync(h->f, 0, fbytes, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, (size_t)gplane, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->status, 0, sizeof(int), h->stream);
@@ -695,20 +702,20 @@ lbm_status lbm_set_flags(lbm_handle h, const uint8_t* flags, int on_device) {
     CUDA_TRY(h, cudaMemcpyAsync(tmp, flags, (size_t)n, cudaMemcpyHostToDevice, h->stream));
     src = tmp;
   }
-  int* bad = nullptr;
-  CUDA_TRY(h, cudaMallocAsync((void**)&bad, sizeof(int), h->stream));
-  CUDA_TRY(h, cudaMemsetAsync(bad, 0, sizeof(int), h->stream));
+  int* seen = nullptr;
+  CUDA_TRY(h, cudaMallocAsync((void**)&seen, 2 * sizeof(int), h->stream));
+  CUDA_TRY(h, cudaMemsetAsync(seen, 0, 2 * sizeof(int), h->stream));
   const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 32);
-  k_flags_in<<<blocks, 256, 0, h->stream>>>(src, h->flags, h->nx, h->ny, h->nz + 2 * h->zg, h->nxp, bad);
+  k_flags_in<<<blocks, 256, 0, h->stream>>>(src, h->flags, h->nx, h->ny, h->nz + 2 * h->zg, h->nxp, seen);
   CUDA_TRY(h, cudaGetLastError());
-  int nbad = 0;
-  CUDA_TRY(h, cudaMemcpyAsync(h->status_host, bad, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaFreeAsync(bad, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(h->seen_host, seen, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaFreeAsync(seen, h->stream));
   if (tmp) CUDA_TRY(h, cudaFreeAsync(tmp, h->stream));
   lbm_status s = launch_classify(h);
   if (s != LBM_OK) return s;
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  nbad = *h->status_host;
+  const int nbad = h->seen_host[0];
+  h->solids = h->seen_host[1] != 0;
   if (nbad) return fail(h, LBM_EINVAL, "%d flag values outside {0,1,2} (stored as solid)", nbad);
   return LBM_OK;
 }
@@ -932,19 +939,32 @@ static bool graph_ready(lbm_handle h) {
 // On small lattices the steps are launch-bound even as graph replays: lbm_step runs them as
 // cooperative launches of k_step_multi, MULTI_CHUNK steps at most each, once the state is
 // steady (as for the graphs).  The line, in row segments of 32 cells against the warps that are
-// resident at once (cap: 32 per SM for D3Q19, 16 for D3Q27, by registers): AA up to one segment
-// per warp (above that the graph's own-cell steps keep the one array in L2 just as well), pull up
-// to two.  Half storage with the split pull step: a quarter, as its graphs run the x-pair kernel.
-// Measured on GB300 (us per step, multi / graph): D3Q19 FP32 AA 64x32x32 4.5 / 6.0, 96x48x32
-// 6.4 / 7.6, 128x48x32 9.6 / 8.7, 64^3 11.4 / 10.3; pull 64x32x32 4.2 / 7.3, 96x48x32 5.9 / 9.0,
-// 128x48x32 9.3 / 10.1, 64^3 10.6 / 12.4, 128x64x64 17.3 / 17.7; FP16 AA 64x32x32 5.8 / 11.1, pull
-// 64x32x32 6.5 / 5.7, 64^3 14.0 / 8.2; D3Q27 FP32 tunnel 64x48x40 AA 12.7 / 10.8, pull 11.7 / 12.6.
+// resident at once (cap: 32 per SM for D3Q19, 24 for D3Q27):
+//  - With boundary cells a graph's step waits for the warps that resolve them: AA up to one segment
+//    per warp, pull up to two (D3Q27 half storage, with more of its time in them, one).
+//  - A periodic box without solid cells has none: up to 16 segments per SM.
+//  - Half storage whose graphs run x-pairs: the split pull step is far ahead with boundary cells in
+//    the list (8 and 4 segments per SM) and behind without (its y/z wraps are listed all the same:
+//    cap); D3Q19 AA in a box up to cap.
+// Measured on GB300 (us per step, multi / graph).  With walls: D3Q19 FP32 AA 64x32x32 4.6 / 6.2, 100x40x30
+// 6.1 / 8.0, 64^3 9.1 / 10.0; pull 64x32x32 4.3 / 7.5, 64^3 9.1 / 12.2, 128x48x48 9.5 / 12.5; FP16 AA
+// 64x32x32 5.7 / 9.3; FP16 pull 64x25x20 6.4 / 5.4; FP16 MRT pull 128x48x48 13.0 / 13.8; D3Q27 FP32 AA 17x60x60
+// 7.4 / 10.3, 32x64x72 11.2 / 9.9; pull 32x64x72 10.3 / 11.8; FP16 regularised pull 17x60x60 10.6 / 11.3,
+// 32x64x72 16.5 / 11.0.  Boxes: D3Q19 FP32 AA 64x32x32 3.4 / 3.6, 64x40x38 4.0 / 3.9, 64x50x46 5.4 / 4.9; pull
+// 64x40x38 4.1 / 3.9, 64^3 8.4 / 7.4; FP16 AA 64x50x46 4.7 / 4.9; FP16 pull 64x32x32 3.5 / 5.7, 64x50x46 5.0 /
+// 6.2; D3Q27 FP32 64x32x32 4.2 / 4.4, 64x50x46 7.2 / 6.2; FP16 pull 64x40x38 4.7 / 8.0.
 // A device that refuses the cooperative launch falls back to the graphs.
 static bool multi_fits(const lbm_s* h) {
   const long long segments = (long long)(h->nxp / 32) * h->ny * h->nz;
-  const long long cap = (h->q == 19 ? 32ll : 16ll) * h->nsm;
-  if (h->prm.streaming != LBM_PULL) return segments <= cap;
-  return segments <= (kparams(h).split ? cap / 4 : 2 * cap);
+  const long long cap = h->q == 19 ? multi_cap<19>(h->nsm) : multi_cap<27>(h->nsm), box = 16ll * h->nsm;
+  bool boundary = h->solids;
+  for (int f = 0; f < 6; f++)
+    boundary = boundary || (h->prm.face_bc[f] != LBM_FACE_PERIODIC && h->prm.face_bc[f] != LBM_FACE_HALO);
+  const bool half = h->prm.precision != LBM_F32;
+  if (h->prm.streaming != LBM_PULL)
+    return segments <= (boundary || (h->q == 19 && half && h->prm.collision == LBM_COLL_TRT) ? cap : box);
+  if (kparams(h).split) return segments <= (boundary ? (h->q == 19 ? 8ll : 4ll) * h->nsm : cap);
+  return segments <= (!boundary ? box : h->q == 27 && half ? cap : 2 * cap);
 }
 
 constexpr int64_t MULTI_CHUNK = 4096;
