@@ -94,8 +94,12 @@ static void step_mode_s(const KParams& p, int closure, const Launch& L, int coll
       return;
     }
   }
-  // half storage: x-pairs, 64 x per warp (D3Q27: the AA even step only, see above)
-  if (sizeof(S) == 2 && ((Q == 19 && (STORE != 1 || odd_pairs(p))) || STORE == 0)) {
+  // half storage: x-pairs, 64 x per warp; D3Q27 (the AA even step only, see above) for rows of more
+  // than 32 cells and lattices of more than a wave of one-cell blocks: below, half the lanes idle or the
+  // longer chain of a pair shows (graph replays of AA, us a step, pairs / one cell: channel 32x80x90
+  // 12.9 / 12.1, 64x50x46 10.3 / 9.8, box 32x64x72 6.4 / 5.7, 17x60x60 5.7 / 4.9).
+  const bool pairs27 = p.nxp > 32 && (long long)L.grid.x * L.grid.y * L.grid.z > (long long)WAVE_CELLS * L.nsm;
+  if (sizeof(S) == 2 && (Q == 19 ? STORE != 1 || odd_pairs(p) : STORE == 0 && pairs27)) {
     if constexpr (sizeof(S) == 2 && (Q == 19 || STORE == 0)) {
       dim3 g = L.grid;
       g.x = (p.nxp + 63) / 64;
