@@ -216,13 +216,12 @@ cudaError_t launch_step_mlp(const KParams& p, int mode, cudaStream_t stream, int
   }
 }
 
-// Blocks of k_row_sums.  EX_SUM: one wave of what is resident (8 per SM).  EX_STATS: four times as
-// many, since a block's rows are all of one plane and those of a wall plane take several times as
-// long (256x128x130 channel: 111 us with one wave; four take 25 us off a pass of two steps, sums,
-// statistics and exports).
-#ifndef LBM_ROW_BLOCKS
-#define LBM_ROW_BLOCKS (8 * 152)
-#endif
+// Blocks of k_row_sums.  EX_SUM: one wave of what is resident (8 per SM), in gathered layouts of more
+// rows two (768x192x192 FP16 D3Q27 tunnel 830 -> 743 us; 96x64x48 channel 36 -> 43 us).  EX_STATS: at least four
+// times as many, in gathered layouts of at most ROWS_MAX rows, since a block's rows are all of one plane
+// and those of a wall plane take several times as long (256x128x130 channel: 111 us with one wave; four take 25 us
+// off a pass of two steps, sums, statistics and exports).
+constexpr int ROW_BLOCKS_SM = 8, ROWS_MAX = 4;
 
 template <int Q, class S, int PAR>
 static void export_par(const KParams& p, int mode, const ExportArgs& a, const Launch& L) {
@@ -240,14 +239,16 @@ static void export_par(const KParams& p, int mode, const ExportArgs& a, const La
       }
       break;
     case EX_SUM: {
-      const int rows = p.ny * p.nz, cnt = (rows + LBM_ROW_BLOCKS - 1) / LBM_ROW_BLOCKS;
+      const int rows = p.ny * p.nz, wave = ROW_BLOCKS_SM * L.nsm;
+      const int want = PAR != 0 && rows >= 4 * wave ? 2 * wave : wave, cnt = (rows + want - 1) / want;
       const int nblk = (rows + cnt - 1) / cnt;
       k_row_sums<Q, S, PAR, EX_SUM><<<(unsigned)nblk, ROW_THREADS, 0, L.stream>>>(p, cnt, a.partial);
       k_row_total<EX_SUM><<<1, 256, 0, L.stream>>>(a.partial, p.ny, nblk, a.sums);
       break;
     }
     default: {
-      const int per = std::max(1, 4 * LBM_ROW_BLOCKS / p.ny);  // blocks per plane
+      const int least = PAR == 0 ? 1 : (p.nz + ROWS_MAX - 1) / ROWS_MAX;
+      const int per = std::max(least, 4 * ROW_BLOCKS_SM * L.nsm / p.ny);  // blocks per plane
       const int cnt = (p.nz + per - 1) / per, nblk = (p.nz + cnt - 1) / cnt * p.ny;
       k_row_sums<Q, S, PAR, EX_STATS><<<(unsigned)nblk, ROW_THREADS, 0, L.stream>>>(p, cnt, a.partial);
       k_row_total<EX_STATS><<<(unsigned)p.ny, 256, 0, L.stream>>>(a.partial, p.ny, nblk, a.sums);

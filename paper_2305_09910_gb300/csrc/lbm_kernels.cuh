@@ -1697,14 +1697,15 @@ __global__ void __launch_bounds__(128) k_export(const __grid_constant__ KParams 
   }
 }
 
-// Sums over fluid cells, in two passes.  k_row_sums: a block takes `cnt` rows, its warps the
+// Sums over fluid cells, in two passes.  k_row_sums: a block takes up to `cnt` rows, its warps the
 // 32-cell segments of these in turn; a lane sums its cells by two_sum, a warp its lanes likewise, and
-// the block's warps in FP64 go to partial[block K + k].  k_row_total then adds the blocks in FP64:
+// the block's warps in FP64 go to partial[block K + k] (EX_STATS: block = chunk ny + plane).  k_row_total
+// then adds the blocks in FP64:
 //   EX_SUM   (K = 5: count, drho, j_x, j_y, j_z) -> sums[0] = count + sum drho = sum rho,
 //            sums[1..3] = sum j = sum rho u (j includes F/2, so u = j / rho);
 //   EX_STATS (K = 10: count, u_x, u_y, u_z, u_x^2, u_y^2, u_z^2, u_x u_y, u_x u_z, u_y u_z)
 //            -> sums[y * 10 + k] += sum over the x-z plane y; the block's rows are then rows of
-//            plane y = block % ny.
+//            one plane.
 // Bound by HBM (one read of the state).  FP64 runs at 1/64 of the FP32 rate here: ten FP64 warp
 // reductions per warp took as long as reading ten rows, hence two_sum and one wave of blocks.
 // 256x128x130 D3Q19 FP32 after a step, both passes: EX_SUM 192 -> 70 us, EX_STATS 275 -> 95
@@ -1721,16 +1722,32 @@ __global__ void __launch_bounds__(ROW_THREADS, 8) k_row_sums(const __grid_consta
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int wpr = p.nxp / 32;
   const int rows = p.ny * p.nz;
-  // rows row0, row0 + rstep, ... of the lattice (row = z ny + y)
-  const int row0 = MODE == EX_STATS ? (blockIdx.x / p.ny) * cnt * p.ny + blockIdx.x % p.ny : blockIdx.x * cnt;
-  const int rstep = MODE == EX_STATS ? p.ny : 1;
+  // Row i of the block (row = z ny + y): row0 + i rstep; in gathered layouts, where the cells of a face
+  // plane take several times as long, dealt out.  EX_SUM: one of every gridDim.x rows, moved on by 37 each
+  // time, as the rows of a z face plane made one block's work and those of a y face one of several blocks'
+  // where gridDim.x is a multiple of ny (512x128x128 FP16 tunnel, both passes: D3Q19 575 -> 183 us, D3Q27
+  // 790 -> 270).  EX_STATS: the planes y = 0 and ny - 1 come first in launch order; as the last blocks they
+  // left a tail (SMs active for 60 % of the FP16 kernel; 768x192x192 channel D3Q19 761 -> 407 us, D3Q27
+  // 1039 -> 505).
+  constexpr bool DEAL = PAR != 0, DEAL_SUM = DEAL && MODE == EX_SUM;
+  int row0 = blockIdx.x * cnt, rstep = 1, slot = blockIdx.x;
+  if (MODE == EX_STATS) {
+    rstep = p.ny;
+    row0 = (blockIdx.x / p.ny) * cnt * p.ny + blockIdx.x % p.ny;
+    if (DEAL) {
+      const int per = gridDim.x / p.ny, o = blockIdx.x / per, chunk = blockIdx.x - o * per;
+      const int y = o == 0 ? 0 : o == 1 ? p.ny - 1 : o - 1;
+      row0 = chunk * cnt * p.ny + y;
+      slot = chunk * p.ny + y;
+    }
+  }
   float hi[K], lo[K];
 #pragma unroll
   for (int k = 0; k < K; k++) hi[k] = lo[k] = 0.f;
   int i = warp / wpr, xw = warp - i * wpr;  // row of the block, segment of the row
   const int di = NW / wpr, dx = NW - di * wpr;
-  while (i < cnt && row0 + i * rstep < rows) {
-    const int row = row0 + i * rstep;
+  while (i < cnt && (DEAL_SUM || row0 + i * rstep < rows)) {
+    const int row = DEAL_SUM ? (int)(i * gridDim.x + (blockIdx.x + 37u * i) % gridDim.x) : row0 + i * rstep;
     const int z = row / p.ny, y = row - z * p.ny, x = xw * 32 + lane;
     i += di;
     xw += dx;
@@ -1738,6 +1755,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 8) k_row_sums(const __grid_consta
       xw -= wpr;
       i++;
     }
+    if (DEAL_SUM && row >= rows) continue;  // (a warp takes or leaves a row as one)
     const int cell = cidx(p, x, y, z);
     float f[Q];
     unsigned outmask = 0;
@@ -1777,7 +1795,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 8) k_row_sums(const __grid_consta
     double t = 0.0;
 #pragma unroll
     for (int w = 0; w < NW; w++) t += red[k][w];
-    partial[(long long)blockIdx.x * K + k] = t;
+    partial[(long long)slot * K + k] = t;
   }
 }
 
