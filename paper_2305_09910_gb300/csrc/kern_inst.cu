@@ -230,13 +230,18 @@ static void export_par(const KParams& p, int mode, const ExportArgs& a, const La
     case EX_MOM:
       // half storage: two cells per thread (64-bit stores need even rows and 8-byte aligned arrays),
       // D3Q27 in natural layout only: gathered, its 80 registers cost more than the pairs give
-      // (FP16 512x256x128 AA after an even step 253 -> 179 us, pull 283 us against 303)
+      // (FP16 512x256x128 AA after an even step 253 -> 179 us, pull 283 us against 303); gathered D3Q19
+      // above a hundred one-cell blocks per SM: below, the lanes with boundary cells, loaded out of line,
+      // make the launch (pull channel, pairs / one cell: 64x32x32 12.9 / 8.5, 128x128x100 (12,800 blocks)
+      // 32-33 / 32, 192x128x100 (19,200) 44.4 / 45.9, 256x200x200 126 / 145)
       if constexpr (sizeof(S) == 2 && (Q == 19 || PAR == 0)) {
-        const int vec = p.nx % 2 == 0 && (uintptr_t)a.rho % 8 == 0 && (uintptr_t)a.u % 8 == 0;
-        k_moments_h2<Q, S, PAR><<<dim3((p.nxp + 63) / 64, L.grid.y, L.grid.z), L.block, 0, L.stream>>>(p, a, vec);
-      } else {
-        k_export<Q, S, PAR, EX_MOM><<<L.grid, L.block, 0, L.stream>>>(p, a);
+        if (PAR == 0 || (long long)L.grid.x * L.grid.y * L.grid.z > 100ll * L.nsm) {
+          const int vec = p.nx % 2 == 0 && (uintptr_t)a.rho % 8 == 0 && (uintptr_t)a.u % 8 == 0;
+          k_moments_h2<Q, S, PAR><<<dim3((p.nxp + 63) / 64, L.grid.y, L.grid.z), L.block, 0, L.stream>>>(p, a, vec);
+          break;
+        }
       }
+      k_export<Q, S, PAR, EX_MOM><<<L.grid, L.block, 0, L.stream>>>(p, a);
       break;
     case EX_SUM: {
       const int rows = p.ny * p.nz, wave = ROW_BLOCKS_SM * L.nsm;
