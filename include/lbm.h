@@ -48,11 +48,14 @@
  * scratch), allocated on the handle's stream.  The caller owns every pointer it passes in.
  * All device work is ordered on the handle's stream (lbm_params.stream, a cudaStream_t;
  * NULL = legacy default stream).  Calls that return data to host memory synchronise that
- * stream before returning.  Host arrays (on_device = 0) in pinned (page-locked) or managed
- * memory are read or written by the kernels in place; an input array there must stay
- * unchanged until the stream has passed the call (as for any asynchronous copy from pinned
- * memory).  Pageable host arrays are staged through device copies.  A handle must not be
- * used from two threads at once.
+ * stream before returning.  Step and transfer kernels let the next launch on the stream begin
+ * early if it asks for that (programmatic stream serialisation): a caller's kernel launched so
+ * has to wait (griddepcontrol.wait, cudaGridDependencySynchronize) before it reads what they
+ * write; any other launch, copy or event is ordered after them as usual.  Host arrays (on_device
+ * = 0) in pinned (page-locked) or managed memory are read or written by the kernels in place; an
+ * input array there must stay unchanged until the stream has passed the call (as for any
+ * asynchronous copy from pinned memory).  Pageable host arrays are staged through device copies.
+ * A handle must not be used from two threads at once.
  *
  * Errors: every call returns an lbm_status; lbm_last_error() gives a message for the last
  * failing call on a handle.  A status of LBM_EUNSTABLE (a non-finite or non-positive
@@ -249,10 +252,13 @@ lbm_status lbm_init_equilibrium(lbm_handle h, const float* rho, const float* u, 
  * rules, fused into one sweep over the lattice per step (the stream-collide kernel of Sec. 3
  * and 5.2, bounded by memory bandwidth).  Asynchronous: returns
  * after enqueuing; instability is reported by lbm_sync.  Once the state is steady, several
- * steps go into one launch: on small lattices (for D3Q19 about 155,000 cells in AA and 310,000
- * in two-grid pull, half of that for D3Q27) cooperative launches of up to 4096 steps separated
+ * steps go into one launch: on small lattices cooperative launches of up to 4096 steps separated
  * by grid-wide barriers, above that, up to 2^22 padded cells, replays of a CUDA graph of 8
  * steps, and single launches on larger lattices; the result has the bits of n single steps.
+ * (The first line on 152 SMs, in padded cells of a lattice with walls, other faces or solid cells: D3Q19
+ * about 155,000 in AA and 310,000 in two-grid pull, D3Q27 117,000 and 230,000, in half storage
+ * 117,000; half-storage pull with the TRT collision 39,000 and 19,000.  A periodic box of fluid cells:
+ * 78,000; in half storage with TRT, pull, or AA of D3Q19, 155,000 and for D3Q27 pull 117,000.)
  * LBM_ECUDA on a handle that lbm_sync has declared unusable. */
 lbm_status lbm_step(lbm_handle h, int64_t n);
 

@@ -58,8 +58,9 @@ enum : int { FACE_PERIODIC = 0, FACE_WALL = 1, FACE_FREESLIP = 2, FACE_INFLOW = 
 enum : int { CLS_INTERIOR = 0, CLS_BOUNDARY = 1, CLS_SKIP = 2, CLS_WRAP = 3 };
 // Class byte = class | CLS_XFACE: a boundary cell on an inflow (-x) or outflow (+x) face whose
 // only rules are those of the directions crossing that face (every other source a fluid cell
-// inside the lattice).  The split half-storage pull step updates such cells in its x-pair
-// kernel; everywhere else they are plain boundary cells (cls_at drops the bit).
+// inside the lattice).  The one-cell steps and the multi-step launch gather and store such cells by
+// gather_xface and store_xface, the pair loads by the former, and the split half-storage pull step
+// updates them in its x-pair kernel; for the exports and sums they are plain boundary cells (cls_at drops the bit).
 constexpr int CLS_MASK = 0x0f, CLS_XFACE = 0x10;
 
 // The split half-storage pull step (x-pair kernel over interior cells + k_step_list) for D3Q27
@@ -679,7 +680,7 @@ __device__ __forceinline__ float rcp_approx(float a) {
 // GELU in its erf form, x Phi(x), for one value or two (packed FP32x2): Phi as a logistic function
 // of an odd polynomial, Phi(x) = 1 / (1 + 2^(x P(x^2))), P of degree 6 fitted to
 // -log2(Phi / (1 - Phi)) / x on |x| <= 6 with weights x^2 Phi (1 - Phi) (the derivative of x Phi by
-// the argument), minimax by reweighted least squares: 6.8e-8 absolute in x Phi.  P is below -2.3
+// the argument), minimax by reweighted least squares: 7.0e-8 absolute in x Phi.  P is below -2.3
 // for every x^2, so the tails go to x and -0.  In float32 over |x| <= 8: largest error 5.9e-7 (half
 // an ulp of x near 8), root mean square 9.3e-8 (1.7e-7 by formula 7.1.26 of Abramowitz & Stegun, which
 // takes four to five more instructions per pair and two divisions instead of two reciprocals).
