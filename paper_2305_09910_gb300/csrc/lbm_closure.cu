@@ -284,7 +284,12 @@ struct BackArgs {
   float k;               // C_s0^2 / ln 2
   float* grad;           // MLP_NPARAM, zeroed before; added to (FP32 atomics)
   double* sums;          // BW_LOSS: [sum w, sum w r^2, loss, blocks done], the first two and the last zeroed
+  int slot;              // (before and after); or null and the slot of call_scratch
 };
+
+// Scratch slots of lbm_closure_loss_grad (see CallScratch), zero between calls but for the loss.
+constexpr int SCRATCH_SLOTS = 64, SCRATCH_DOUBLES = 4;
+__device__ double call_scratch[SCRATCH_SLOTS * SCRATCH_DOUBLES];
 
 constexpr int BW_MINB = 2;          // resident blocks per SM: 255 registers (3 blocks spill 0.6 KB and ran 20 % slower)
 constexpr int BW_WARPS = 4;         // warps per block
@@ -543,22 +548,27 @@ __global__ void __launch_bounds__(32 * BW_WARPS, BW_MINB) k_mlp_backward(const _
     atomicAdd(a.grad + e, g);
   }
   if (MODE != BW_LOSS) return;
+  double* const sums = a.sums ? a.sums : call_scratch + a.slot * SCRATCH_DOUBLES;
   if (tid < 2) {
     double v = 0.0;
     for (int w = 0; w < BW_WARPS; w++) v += sm.red[tid][w];
-    atomicAdd(a.sums + tid, v);
+    atomicAdd(sums + tid, v);
   }
   // the last block to finish divides by the sum of the weights
   __threadfence();
   __syncthreads();
-  if (tid == 0) sm.last = atomicAdd(reinterpret_cast<unsigned*>(a.sums + 3), 1u) == gridDim.x - 1;
+  if (tid == 0) sm.last = atomicAdd(reinterpret_cast<unsigned*>(sums + 3), 1u) == gridDim.x - 1;
   __syncthreads();
   if (!sm.last) return;
   __threadfence();
-  const double wsum = __ldcg(a.sums), wrr = __ldcg(a.sums + 1);
+  const double wsum = __ldcg(sums), wrr = __ldcg(sums + 1);
   const float inv = wsum > 0.0 ? (float)(1.0 / wsum) : 0.f;
   for (int e = tid; e < MLP_NPARAM; e += 32 * BW_WARPS) a.grad[e] = __ldcg(a.grad + e) * inv;
-  if (tid == 0) a.sums[2] = wsum > 0.0 ? wrr / wsum : 0.0;
+  __syncthreads();  // all threads have read the sums
+  if (tid == 0) {
+    sums[0] = sums[1] = sums[3] = 0.0;
+    sums[2] = wsum > 0.0 ? wrr / wsum : 0.0;
+  }
 }
 
 __global__ void k_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1,
@@ -672,43 +682,41 @@ lbm_status lbm_closure_samples(lbm_handle fine, double tau0_c, double cs0, const
   return LBM_OK;
 }
 
-// Scratch of a call that synchronises before it returns: one of SLOTS small blocks in the module's
-// own device storage, taken for the duration of the call by any thread and stream, or stream-ordered
-// memory where all are taken.  An allocation per call cost 0.1 ms: the default pool gives its memory
-// back at every synchronisation and maps 32 MB again.  The storage lives and dies with the module in
-// its context, and its address is asked for by every call: after a device reset a kept one is stale.
-constexpr int SCRATCH_SLOTS = 64, SCRATCH_DOUBLES = 4;
-__device__ double call_scratch[SCRATCH_SLOTS * SCRATCH_DOUBLES];
-
+// Scratch of a call that synchronises before it returns: one of SCRATCH_SLOTS small blocks in the
+// module's own device storage, taken for the duration of the call by any thread and stream, or
+// stream-ordered memory where all are taken.  An allocation per call cost 0.1 ms: the default pool gives
+// its memory back at every synchronisation and maps 32 MB again.  The storage lives and dies with the
+// module in its context and the host keeps no address of it (after a device reset that would be stale);
+// the kernel finds the slot itself and leaves it zeroed, so a call asks for no address and zeroes nothing.
 class CallScratch {
  public:
   cudaError_t take(cudaStream_t st) {
-    void* mem = nullptr;
     cudaError_t e = cudaGetDevice(&dev_);
-    if (e == cudaSuccess) e = cudaGetSymbolAddress(&mem, call_scratch);
     if (e != cudaSuccess) return e;
     if (dev_ < DEVICES) {
       std::lock_guard<std::mutex> hold(lock());
-      for (int i = 0; slot_ < 0 && i < SCRATCH_SLOTS; i++)
+      for (int i = 0; slot < 0 && i < SCRATCH_SLOTS; i++)
         if (!(used()[dev_] >> i & 1)) {
           used()[dev_] |= 1ull << i;
-          slot_ = i;
-          p = static_cast<double*>(mem) + i * SCRATCH_DOUBLES;
+          slot = i;
         }
     }
-    return p ? cudaSuccess : cudaMallocAsync((void**)&p, SCRATCH_DOUBLES * sizeof(double), st);
+    if (slot >= 0) return cudaSuccess;
+    e = cudaMallocAsync((void**)&p, SCRATCH_DOUBLES * sizeof(double), st);
+    return e == cudaSuccess ? cudaMemsetAsync(p, 0, SCRATCH_DOUBLES * sizeof(double), st) : e;
   }
   // after the call's work is queued; idle: the stream has been waited for
   void give(cudaStream_t st, bool idle) {
-    if (slot_ < 0) {
+    if (slot < 0) {
       if (p) cudaFreeAsync(p, st);
     } else if (idle) {  // after an error the slot stays taken: its work may still be running
       std::lock_guard<std::mutex> hold(lock());
-      used()[dev_] &= ~(1ull << slot_);
+      used()[dev_] &= ~(1ull << slot);
     }
     p = nullptr;
   }
   double* p = nullptr;
+  int slot = -1;
 
  private:
   static constexpr int DEVICES = 64;
@@ -720,7 +728,7 @@ class CallScratch {
     static uint64_t u[DEVICES];
     return u;
   }
-  int dev_ = 0, slot_ = -1;
+  int dev_ = 0;
 };
 
 lbm_status lbm_mlp_forward(const float* params, const float* x, int64_t n, float* y, void* stream) {
@@ -793,8 +801,6 @@ lbm_status lbm_closure_loss_grad(const float* params, const float* x, const floa
   unsigned grid = 0;
   cudaError_t e = backward_grid(n, &grid);
   if (e == cudaSuccess) e = scratch.take(st);
-  double* const sums = scratch.p;
-  if (e == cudaSuccess) e = cudaMemsetAsync(sums, 0, SCRATCH_DOUBLES * sizeof(double), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, MLP_NPARAM * sizeof(float), st);
   if (e == cudaSuccess && n > 0) {
     BackArgs a{};
@@ -808,11 +814,17 @@ lbm_status lbm_closure_loss_grad(const float* params, const float* x, const floa
     a.stride = stride;
     a.k = (float)(cs0 * cs0 / std::log(2.0));
     a.grad = grad;
-    a.sums = sums;
+    a.sums = scratch.p;
+    a.slot = scratch.slot;
     k_mlp_backward<BW_LOSS><<<grid, 32 * BW_WARPS, sizeof(BackSmem), st>>>(a);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(loss, sums + 2, sizeof(double), cudaMemcpyDefault, st);
+  static const double zero = 0.0;
+  if (e == cudaSuccess && n == 0) e = cudaMemcpyAsync(loss, &zero, sizeof(double), cudaMemcpyDefault, st);
+  else if (e == cudaSuccess && scratch.p) e = cudaMemcpyAsync(loss, scratch.p + 2, sizeof(double), cudaMemcpyDefault, st);
+  else if (e == cudaSuccess)
+    e = cudaMemcpyFromSymbolAsync(loss, call_scratch, sizeof(double), (scratch.slot * SCRATCH_DOUBLES + 2) * sizeof(double),
+                                  cudaMemcpyDefault, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   scratch.give(st, e == cudaSuccess);
   if (e != cudaSuccess) {

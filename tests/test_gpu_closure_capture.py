@@ -89,3 +89,25 @@ print("ok")
 def test_scratch_of_the_loss_gradient(program):
     r = subprocess.run([sys.executable, "-c", program], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), (r.returncode, r.stdout[-500:], r.stderr[-2000:])
+
+
+def test_scratch_slots_are_left_as_they_were_found():
+    """Calls in a row, of different sizes and of no sample, and with all weights zero between: a slot holds
+    nothing of the call before."""
+    import torch
+
+    from paper_2305_09910_gb300 import lbm
+
+    g = torch.Generator(device="cuda").manual_seed(9)
+    n = 5000
+    p = torch.randn(1345, device="cuda", generator=g) * 0.1
+    x = torch.randn(n, 7, device="cuda", generator=g)
+    s, t, w = (torch.rand(n, device="cuda", generator=g) for _ in range(3))
+    grad, dev = torch.zeros(1345, device="cuda"), torch.zeros(1, device="cuda", dtype=torch.float64)
+    first = {}
+    for k in range(3):
+        for m in (5000, 1, 0, 33, 640):
+            loss = lbm.lbm_closure_loss_grad(p, x, t, s, w, m, 0, 1, 0.1, grad)
+            assert abs(loss - first.setdefault(m, loss)) <= 1e-12 * first[m]  # float64 sums in another order
+            assert lbm.lbm_closure_loss_grad(p, x, t, s, 0 * w, m, 0, 1, 0.1, grad) == 0.0
+    assert first[0] == 0.0 and first[5000] > 0.0
